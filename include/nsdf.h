@@ -297,7 +297,7 @@ nsdf_status nsdf_set_grouped_config(nsdf_ctx *ctx, int points_per_thread,
  * (float, DEVICE, n^3 values; n = 256 is 64 MB).
  *
  * nsdf_voxel_build fills the grid with the exact signed distance of every
- * node to a watertight mesh (the brute force of nsdf_mesh_sdf; same mesh
+ * node to a watertight mesh (as nsdf_mesh_sdf; same mesh
  * arguments, DEVICE pointers).  n in [2, 2048].
  *
  * nsdf_voxel_collide answers the collision query of nsdf_collide from the
@@ -320,14 +320,18 @@ nsdf_status nsdf_voxel_collide(const float *grid, int n, const float *lo,
                                uint8_t *out_hit, nsdf_stream stream);
 
 /*
- * Ground-truth signed distance to a watertight triangle mesh by brute force
+ * Ground-truth signed distance to a watertight triangle mesh
  * (the targets of Sec. 3.1): out_sdf[i] = +-min_t dist(p_i, triangle t),
  * negative where the generalized winding number exceeds 1/2 (interior
  * negative, Sec. 3.2).  verts: float [n_verts*3]; faces: int32 [n_faces*3],
  * counter-clockwise seen from outside; pts float4; all device pointers (a
  * host array: NSDF_ERR_INVALID_ARG, nothing is launched).
- * The winding number is accumulated in FP32 and recomputed in FP64 for
- * points with |w - 1/2| < 0.25 or distance < 1e-3.
+ * A closed mesh of at least 128 faces is answered through a bounding-box tree
+ * that each call builds in stream-ordered scratch memory; its winding number is
+ * the signed count of the faces a ray crosses.  Other meshes, calls recorded
+ * into a CUDA graph and calls for which no scratch memory is left evaluate every
+ * face for every point: the winding number is then accumulated in FP32 and
+ * recomputed in FP64 for points with |w - 1/2| < 0.25 or distance < 1e-3.
  */
 nsdf_status nsdf_mesh_sdf(const float *verts, int64_t n_verts,
                           const int32_t *faces, int64_t n_faces,

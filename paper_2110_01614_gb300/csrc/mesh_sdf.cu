@@ -1,6 +1,7 @@
-// Brute-force exact signed distance to a watertight triangle mesh: the
-// ground truth a network is fitted to (Sec. 3.1) and the plain reference a
-// cloth run can collide against.
+// Exact signed distance to a watertight triangle mesh: the ground truth a
+// network is fitted to (Sec. 3.1) and the plain reference a cloth run can
+// collide against.  Closed meshes of 128 faces and more go through the tree of
+// mesh_tree.cu; this is the brute force for the others and the dispatch.
 //
 // Per point: unsigned distance = min over triangles of the distance to the
 // triangle's closest point (barycentric Voronoi-region test: vertex, edge or
@@ -15,6 +16,7 @@
 // angle is ill-conditioned) the warp recomputes w in FP64, all 32 lanes
 // splitting the triangles of one such point at a time.
 
+#include "mesh_tree.cuh"
 #include "nsdf_internal.h"
 
 namespace nsdf {
@@ -52,104 +54,21 @@ __device__ void load_chunk(TriChunk &t, const float *__restrict__ V, int64_t nv,
   }
 }
 
-template <typename T>
-struct V3 {
-  T x, y, z;
-};
-template <typename T>
-__device__ __forceinline__ V3<T> sub(V3<T> a, V3<T> b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
-template <typename T>
-__device__ __forceinline__ T dot(V3<T> a, V3<T> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-template <typename T>
-__device__ __forceinline__ V3<T> cross(V3<T> a, V3<T> b) {
-  return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
-}
-
-// Squared distance from p to triangle (a, b, c) by its Voronoi regions.
-__device__ __forceinline__ float tri_dist2(V3<float> p, V3<float> a, V3<float> b, V3<float> c) {
-  const V3<float> ab = sub(b, a), ac = sub(c, a), ap = sub(p, a);
-  const float d1 = dot(ab, ap), d2 = dot(ac, ap);
-  V3<float> q;
-  if (d1 <= 0.f && d2 <= 0.f) {
-    q = a;
-  } else {
-    const V3<float> bp = sub(p, b);
-    const float d3 = dot(ab, bp), d4 = dot(ac, bp);
-    if (d3 >= 0.f && d4 <= d3) {
-      q = b;
-    } else {
-      const float vc = d1 * d4 - d3 * d2;
-      if (vc <= 0.f && d1 >= 0.f && d3 <= 0.f) {
-        const float v = d1 / (d1 - d3);
-        q = {a.x + v * ab.x, a.y + v * ab.y, a.z + v * ab.z};
-      } else {
-        const V3<float> cp = sub(p, c);
-        const float d5 = dot(ab, cp), d6 = dot(ac, cp);
-        if (d6 >= 0.f && d5 <= d6) {
-          q = c;
-        } else {
-          const float vb = d5 * d2 - d1 * d6;
-          if (vb <= 0.f && d2 >= 0.f && d6 <= 0.f) {
-            const float w = d2 / (d2 - d6);
-            q = {a.x + w * ac.x, a.y + w * ac.y, a.z + w * ac.z};
-          } else {
-            const float va = d3 * d6 - d5 * d4;
-            if (va <= 0.f && (d4 - d3) >= 0.f && (d5 - d6) >= 0.f) {
-              const float w = (d4 - d3) / ((d4 - d3) + (d5 - d6));
-              q = {b.x + w * (c.x - b.x), b.y + w * (c.y - b.y), b.z + w * (c.z - b.z)};
-            } else {
-              const float den = 1.f / (va + vb + vc);
-              const float v = vb * den, w = vc * den;
-              q = {a.x + ab.x * v + ac.x * w, a.y + ab.y * v + ac.y * w, a.z + ab.z * v + ac.z * w};
-            }
-          }
-        }
-      }
-    }
-  }
-  const V3<float> d = sub(p, q);
-  return dot(d, d);
-}
-
-template <typename T>
-__device__ __forceinline__ T solid_angle(V3<T> p, V3<T> a, V3<T> b, V3<T> c) {
-  const V3<T> A = sub(a, p), B = sub(b, p), C = sub(c, p);
-  const T la = sqrt(dot(A, A)), lb = sqrt(dot(B, B)), lc = sqrt(dot(C, C));
-  const T num = dot(A, cross(B, C));
-  const T den = la * lb * lc + dot(A, B) * lc + dot(A, C) * lb + dot(B, C) * la;
-  return T(2) * atan2(num, den);
-}
-
-// Points of the implicit grid: node (i, j, k) at lo + (i, j, k) * h, index
-// i + N (j + N k).
-struct GridPts {
-  int n;
-  float lo[3], h[3];
-};
-
 __global__ void __launch_bounds__(kThreads) mesh_sdf_kernel(const float *__restrict__ V, int64_t nv,
                                                             const int32_t *__restrict__ F,
                                                             int64_t nf, const float4 *__restrict__ pts,
                                                             int64_t n, float *__restrict__ out,
-                                                            const GridPts grid) {
+                                                            const GridPts grid,
+                                                            const MeshTreeHeader *tree) {
+  if (tree && mesh_tree_usable(tree)) return;     // the tree kernel has answered
   extern __shared__ float4 smem4[];
   TriChunk &tc = *reinterpret_cast<TriChunk *>(smem4);
   __shared__ double wacc[kThreads / 32][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (idx < n) {
-    if (pts) {
-      p4 = pts[idx];
-    } else {
-      const int64_t N = grid.n;
-      p4.x = grid.lo[0] + grid.h[0] * (float)(idx % N);
-      p4.y = grid.lo[1] + grid.h[1] * (float)((idx / N) % N);
-      p4.z = grid.lo[2] + grid.h[2] * (float)(idx / (N * N));
-    }
-  }
-  const V3<float> p = {p4.x, p4.y, p4.z};
-  float best = 3.4e38f, wsum = 0.f;
+  V3<float> p = {0.f, 0.f, 0.f};
+  if (idx < n) p = query_point(pts, grid, idx);
+  float best = kFarDist2, wsum = 0.f;
   for (int64_t f0 = 0; f0 < nf; f0 += kChunk) {
     __syncthreads();
     load_chunk(tc, V, nv, F, f0, nf);
@@ -218,10 +137,34 @@ cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *
       g.h[c] = h[c];
     }
   }
+  // The tree needs scratch memory, taken from the device's stream-ordered pool
+  // and given back behind the kernels.  Without it (none left, or a stream
+  // that is being captured: the graph stays free of allocations) the
+  // brute-force kernel answers alone.
+  void *mem = nullptr;
+  if (n_faces >= kTreeMinFaces && n_faces <= kTreeMaxFaces) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+        cudaMallocAsync(&mem, mesh_tree_bytes(n_faces, pts ? n : 0), s) != cudaSuccess)
+      mem = nullptr;
+    if (!mem) cudaGetLastError();
+  }
+  if (mem) {
+    e = launch_mesh_tree(verts, n_verts, faces, n_faces, pts, n, out, g, mem, s);
+    if (e != cudaSuccess) {
+      cudaFreeAsync(mem, s);
+      return e;
+    }
+  }
   const int64_t blocks = (n + kThreads - 1) / kThreads;
-  mesh_sdf_kernel<<<(unsigned)blocks, kThreads, smem, s>>>(verts, n_verts, faces, n_faces, pts, n,
-                                                          out, g);
-  return cudaGetLastError();
+  mesh_sdf_kernel<<<(unsigned)blocks, kThreads, smem, s>>>(
+      verts, n_verts, faces, n_faces, pts, n, out, g, static_cast<const MeshTreeHeader *>(mem));
+  e = cudaGetLastError();
+  if (mem) {
+    const cudaError_t e2 = cudaFreeAsync(mem, s);
+    if (e == cudaSuccess) e = e2;
+  }
+  return e;
 }
 
 }  // namespace nsdf

@@ -1,0 +1,41 @@
+// Bounding-box tree over a triangle mesh (mesh_tree.cu), built on the device
+// by every call that uses it.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "mesh_tri.cuh"
+
+namespace nsdf {
+
+// Written by the build, read by the queries.  All zero before the build.
+struct MeshTreeHeader {
+  unsigned neg_lo[3], hi[3];      // bounds of the faces kept, as ordered keys (neg_lo: of -lo)
+  unsigned valid;                 // faces kept (every vertex index in range)
+  unsigned nonfinite;             // a kept face has a NaN or infinite vertex
+  unsigned long long boundary;    // hash of the mesh's boundary: 0 for a closed mesh
+  unsigned done;                  // blocks of the box kernel that have finished
+};
+
+// Can the tree answer for this mesh?  Only a closed mesh of finite vertices
+// has a winding number that ray crossings give.
+__device__ __forceinline__ bool mesh_tree_usable(const MeshTreeHeader *h) {
+  return h->boundary == 0ull && h->nonfinite == 0u && h->valid > 0u;
+}
+
+// Meshes below this take the brute-force kernel, whose one launch costs less
+// than the tree's seven; above the maximum 32-bit heap indices would run out.
+constexpr int64_t kTreeMinFaces = 128;
+constexpr int64_t kTreeMaxFaces = int64_t(1) << 28;
+
+// n_points: explicit query points (0 for a grid, whose nodes need no scratch).
+size_t mesh_tree_bytes(int64_t n_faces, int64_t n_points);
+// Build the tree in `mem` (mesh_tree_bytes, 256-byte aligned) and write the
+// signed distances of all points if it is usable; out is untouched otherwise.
+cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t *faces,
+                             int64_t n_faces, const float4 *pts, int64_t n, float *out,
+                             const GridPts &grid, void *mem, cudaStream_t s);
+
+}  // namespace nsdf

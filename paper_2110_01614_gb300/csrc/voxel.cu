@@ -3,8 +3,8 @@
 // interpolation, against which the network's memory, speed and accuracy are
 // set.
 //
-// Build: every grid node's exact signed distance to the mesh, from the
-// brute-force kernel (mesh_sdf.cu) run over the implicit grid.
+// Build: every grid node's exact signed distance to the mesh, from the mesh
+// kernels (mesh_tree.cu, mesh_sdf.cu) run over the implicit grid.
 // Query (one thread per point, float4 in and out): u = (p - lo) / h clamped
 // to the box; the cell c = min(floor(u), N - 2) and t = u - c; sdf = the
 // trilinear interpolant of the cell's 8 nodes; grad = its analytic gradient
