@@ -30,7 +30,7 @@
 namespace nsdf {
 
 // 32 MiB: 36 CTAs for the 512-wide, 8-layer body-scale network in 16 bits
-// (896 KiB of slopes per CTA), 73 in FP32.
+// (896 KiB of slopes per CTA) and in FP32.
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
 
 __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];

@@ -31,10 +31,17 @@ int fp32_ctas_per_sm(int width, int pt, bool ff) {
   return 1;
 }
 
-// The single-network launch uses 8 points per thread.
+// Tile shape of a single-network launch: the small tiles when all of them fit
+// on the GPU at once in place of the large ones (more SMs at work; they then
+// also need no more scratch than the large shape's grid), else the large.
+static int single_shape(int width, int64_t n, int num_sms, bool ff) {
+  const int P = fp32_tile_points(width, 4);
+  return (n + P - 1) / P <= (int64_t)num_sms * fp32_ctas_per_sm(width, 8, ff) ? 4 : 8;
+}
+
 int query_fp32_grid(int width, int64_t n, int num_sms, bool ff) {
-  const int P = fp32_tile_points(width, 8);
-  if (P == 0) return 0;
+  if (!query_fp32_supported(width)) return 0;
+  const int P = fp32_tile_points(width, single_shape(width, n, num_sms, ff));
   const int64_t tiles = (n + P - 1) / P;
   const int64_t cap = (int64_t)num_sms * fp32_ctas_per_sm(width, 8, ff);
   return (int)(tiles < cap ? (tiles < 1 ? 1 : tiles) : cap);
@@ -62,7 +69,7 @@ cudaError_t launch_query_fp32_grouped(const QueryParams &p, int pt, int grid, cu
 cudaError_t launch_query_fp32(const QueryParams &p, int num_sms, cudaStream_t s) {
   const int grid = query_fp32_grid(p.width, p.n, num_sms, p.ff > 0);
   if (grid == 0) return cudaErrorInvalidValue;
-  return launch_query_fp32_grouped(p, 8, grid, s);
+  return launch_query_fp32_grouped(p, single_shape(p.width, p.n, num_sms, p.ff > 0), grid, s);
 }
 
 }  // namespace nsdf

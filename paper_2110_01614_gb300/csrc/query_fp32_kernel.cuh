@@ -21,40 +21,66 @@
 // sigmoid(beta z_l) of every hidden layer is parked in a per-CTA scratch
 // slab between the forward and the reverse pass; it is written and read by
 // the same thread in a lane-contiguous order (coalesced, L2-resident).
+//
+// Products.  A thread owns 8 points x TC columns (TC = 8 from width 256 on, 4
+// below); a warp covers 32 points x 8 TC columns, a CTA PW x CW warps.  The
+// activation tile is stored [column][point], so a thread reads its points as
+// natural pairs and multiplies each pair by a weight in both lanes of one
+// f32x2 FMA: per k step 2 x 16 bytes of points and TC / 4 x 16 bytes of weights
+// feed 4 TC paired FMAs.  With the scalar form (a warp on one group of 8
+// points, weights read as single words) the issue slots and the shared-memory
+// reads bounded the kernel at 0.54 of the FMA rate; here the FP32 pipe is busy
+// 0.7 of the time (a paired FMA beside the moves that double a weight runs at
+// 0.75-0.88 of the pipe in a probe; scalar FMAs in this layout measure 3-9%
+// slower).  Measured, before -> now: 131,077 points of 3-512x8-1 22.9 -> 17.8 ms,
+// 300,000 of the 8 x 256 Fourier-feature network 16.8 -> 11.5 ms, 1,048,576 of
+// 3-64x3-1 1.23 -> 0.76 ms, 1,000 points of 3-512x8-1 0.85 -> 0.73 ms.
+// Each accumulator is the same chain of FMAs over k, so z, the activations and
+// the slopes keep their bits.  A layer's output replaces its input in place
+// once every warp has read it, which leaves room for tiles of 64 points at
+// width 512 (half the weight traffic of 32); the weight panels of all layers
+// are one stream of chunks through a cp.async ring that runs ahead across the
+// layers' epilogues, with one barrier per chunk.
+//
+// The small shape (PT = 4, half the warps and half the points per tile) is for
+// launches whose small tiles all fit on the GPU at once, where a larger tile
+// would leave SMs idle, and for the grouped launch's tuner.
 
 #pragma once
 
-#include "nsdf_internal.h"
+#include "f32x2.cuh"
 #include "ff_phase.cuh"
+#include "nsdf_internal.h"
 
 namespace nsdf {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr float kInvSqrt2 = 0.70710678118654752f;
 
 template <int W, int PT_ = 8>
 struct Cfg {
-  static constexpr int WG = (W >= 256) ? 2 : 1;   // warps sharing a point group
-  static constexpr int PT = PT_;                   // points per thread (tile shape)
-  static constexpr int GROUPS = kWarps / WG;
-  static constexpr int P = GROUPS * PT;            // points per tile
-  static constexpr int CT = W / (32 * WG);         // columns per thread
-  static constexpr int KC0 = 8192 / W;
-  static constexpr int KC = KC0 > W ? W : (KC0 < 4 ? 4 : KC0);   // panel rows
+  static constexpr int TP = 8;                          // points per thread
+  static constexpr int TC = W >= 256 ? 8 : 4;           // columns per thread
+  static constexpr int CW = W / (8 * TC);               // warps across the columns
+  static constexpr int PW = (W <= 64 ? 4 : 2) / (PT_ == 4 ? 2 : 1);   // warps across the points
+  static constexpr int THREADS = 32 * CW * PW;
+  static constexpr int P = 32 * PW;                     // points per tile
+  static constexpr int XS = P + 4;                      // floats per activation row
+  static constexpr int KC = W == 512 ? 8 : (4096 / W > W ? W : 4096 / W);   // panel rows per chunk
   static constexpr int NCHUNK = W / KC;
-  static_assert(W % (32 * WG) == 0, "width");
-  static_assert(W % KC == 0 && KC % 4 == 0, "panel");
+  static constexpr int NS = (W == 512 && PT_ == 8) ? 3 : 2;                 // ring slots
+  // CTAs per SM that the registers are budgeted for
+  static constexpr int MIN_CTAS = THREADS >= 512 ? 1 : (W >= 128 ? 512 / THREADS : 768 / THREADS);
+  static_assert(W % (8 * TC) == 0 && W % KC == 0 && P <= THREADS, "shape");
   // shared memory carve-up (floats)
   static constexpr int X_OFF = 0;
-  static constexpr int Y_OFF = X_OFF + P * W;
-  static constexpr int M_OFF = Y_OFF + P * W;
-  static constexpr int PS_OFF = M_OFF + 2 * KC * W;          // float4 [P]
-  static constexpr int RED_OFF = PS_OFF + 4 * P;             // [WG][P][4]
-  static constexpr int DIR_OFF = RED_OFF + WG * P * 4;       // [P][4]
+  static constexpr int M_OFF = X_OFF + XS * W;
+  static constexpr int PS_OFF = M_OFF + NS * KC * W;         // float4 [P]
+  static constexpr int RED_OFF = PS_OFF + 4 * P;             // [CW][P][4]
+  static constexpr int DIR_OFF = RED_OFF + CW * P * 4;       // [P][4]
   static constexpr int SMEM_FLOATS = DIR_OFF + 4 * P;
   static constexpr size_t SMEM_BYTES = sizeof(float) * SMEM_FLOATS;
+  static_assert(SMEM_BYTES <= 232448, "shared memory");
 };
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -91,80 +117,36 @@ __device__ __forceinline__ void act_and_slope(float z, float beta, float inv_bet
   }
 }
 
-// Stage rows [k0, k0+KC) of a row-major [W x W] panel into shared memory.
-template <int W, int PT_ = 8>
-__device__ __forceinline__ void stage_panel(float *dst, const float *src, int k0) {
-  using C = Cfg<W, PT_>;
-  constexpr int VEC = C::KC * W / 4;
-  const float4 *s4 = reinterpret_cast<const float4 *>(src + (size_t)k0 * W);
-  float4 *d4 = reinterpret_cast<float4 *>(dst);
-  for (int v = threadIdx.x; v < VEC; v += kThreads) cp_async16(d4 + v, s4 + v);
-  cp_async_commit();
-}
-
-// acc[i][j] = sum_k X[g*PT + i][k] * M[k][col_j] for the thread's PT points
-// and CT columns; M is a global [W x W] row-major panel streamed through
-// two shared buffers.  All threads of the CTA must call this together.
-template <int W, int PT_ = 8>
-__device__ __forceinline__ void panel_product(const float *X, const float *M, float *Ms,
-                                              int g, int colbase,
-                                              float (&acc)[Cfg<W, PT_>::PT][Cfg<W, PT_>::CT]) {
-  using C = Cfg<W, PT_>;
-#pragma unroll
-  for (int i = 0; i < C::PT; ++i)
-#pragma unroll
-    for (int j = 0; j < C::CT; ++j) acc[i][j] = 0.0f;
-  stage_panel<W, PT_>(Ms, M, 0);
-  for (int kc = 0; kc < C::NCHUNK; ++kc) {
-    if (kc + 1 < C::NCHUNK) {
-      stage_panel<W, PT_>(Ms + ((kc + 1) & 1) * C::KC * W, M, (kc + 1) * C::KC);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
-    __syncthreads();
-    const float *Mc = Ms + (kc & 1) * C::KC * W;
-    const float *Xr = X + (g * C::PT) * W + kc * C::KC;
-#pragma unroll 1
-    for (int kk = 0; kk < C::KC; kk += 4) {
-      float4 xv[C::PT];
-#pragma unroll
-      for (int i = 0; i < C::PT; ++i) xv[i] = *reinterpret_cast<const float4 *>(Xr + i * W + kk);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float wv[C::CT];
-#pragma unroll
-        for (int j = 0; j < C::CT; ++j) wv[j] = Mc[(kk + q) * W + colbase + 32 * j];
-#pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          float xs = q == 0 ? xv[i].x : q == 1 ? xv[i].y : q == 2 ? xv[i].z : xv[i].w;
-#pragma unroll
-          for (int j = 0; j < C::CT; ++j) acc[i][j] = fmaf(xs, wv[j], acc[i][j]);
-        }
-      }
-    }
-    __syncthreads();
-  }
+__device__ __forceinline__ float el4(const float4 &v, int i) {
+  return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
 
 // FF: the network has the Fourier-feature input layer (compiled separately,
 // so that networks without it keep the registers, hence the occupancy, of a
 // kernel without that code).
 template <int W, int PT_ = 8, bool FF = false>
-__global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm) {
+__global__ void __launch_bounds__(Cfg<W, PT_>::THREADS, Cfg<W, PT_>::MIN_CTAS)
+    query_fp32_kernel(const __grid_constant__ QueryParams prm) {
   using C = Cfg<W, PT_>;
   extern __shared__ float4 smem4[];
   float *smem = reinterpret_cast<float *>(smem4);
   float *X = smem + C::X_OFF;
-  float *Y = smem + C::Y_OFF;
   float *Ms = smem + C::M_OFF;
   float4 *Ps = reinterpret_cast<float4 *>(smem + C::PS_OFF);
   float *red = smem + C::RED_OFF;
   float *dir = smem + C::DIR_OFF;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = warp / C::WG, part = warp % C::WG;
-  const int colbase = part * (W / C::WG) + lane;
+  const int cw = warp % C::CW, pw = warp / C::CW;
+  // this thread's points: pb .. pb + 3 and pb + 16 .. pb + 19; columns cb .. cb + 3
+  // (and cb + 32 .. cb + 35 when TC = 8)
+  // (lanes that differ in bit 0 share their points, lanes that differ in bit 1
+  // their columns: 16-byte shared loads then merge, two wavefronts instead of four)
+  const int lp = ((lane >> 1) & 1) | ((lane >> 2) & 2),
+            lc = (lane & 1) | ((lane >> 1) & 2) | ((lane >> 2) & 4);
+  const int pb = 32 * pw + 4 * lp, cb = cw * 8 * C::TC + 4 * lc;
+  auto point = [&](int i) { return pb + (i < 4 ? i : 12 + i); };
+  auto column = [&](int j) { return cb + (j < 4 ? j : 28 + j); };
   const int L = prm.n_hidden;
   const int skip = prm.skip;
   const int nshort = W - 3;   // outputs of the layer feeding the skip
@@ -172,10 +154,11 @@ __global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm
   const float inv_beta = 1.0f / prm.beta;
   const bool grouped = prm.g_nets > 0;
   const int64_t ntiles = grouped ? (int64_t)prm.g_tile_start[prm.g_nets] : (prm.n + C::P - 1) / C::P;
-  // per-CTA slope slab: [L-1][PT][CT][kThreads]
-  float *slab = prm.scratch + (size_t)blockIdx.x * (size_t)(L - 1) * C::P * W;
-  auto slot = [&](int l, int i, int j) -> float * {
-    return slab + (((size_t)l * C::PT + i) * C::CT + j) * kThreads + tid;
+  // per-CTA slope slab: [L-1][TC][2][THREADS] float4
+  float4 *slab = reinterpret_cast<float4 *>(prm.scratch) +
+                 (size_t)blockIdx.x * (size_t)(L > 1 ? L - 1 : 1) * (C::P * W / 4);
+  auto slot = [&](int l, int j, int half) -> float4 * {
+    return slab + ((size_t)(l * C::TC + j) * 2 + half) * C::THREADS + tid;
   };
 
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -204,6 +187,32 @@ __global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm
       nvalid = prm.n - base;
     }
     if (nvalid > C::P) nvalid = C::P;
+
+    // ---- the tile's weight panels, in the order they are used, as one stream
+    // of KC-row chunks: (ff0_t), fwd_t 1 .. L-1, bwd L-1 .. 1, (ff0) ----
+    const int nchunks = (2 * (L - 1) + (FF ? 2 : 0)) * C::NCHUNK;
+    auto stage = [&](int q) {
+      if (q < nchunks) {
+        int m = q / C::NCHUNK;
+        const float *src;
+        if (FF && m == 0) {
+          src = ff0_t;
+        } else {
+          if (FF) --m;
+          src = m < L - 1 ? fwd_t + (size_t)m * W * W
+                          : (m < 2 * (L - 1) ? bwdw + (size_t)(2 * (L - 1) - 1 - m) * W * W : ff0);
+        }
+        const float4 *s4 = reinterpret_cast<const float4 *>(src + (size_t)(q % C::NCHUNK) * C::KC * W);
+        float4 *d4 = reinterpret_cast<float4 *>(Ms + (q % C::NS) * C::KC * W);
+#pragma unroll 4
+        for (int v = tid; v < C::KC * W / 4; v += C::THREADS) cp_async16(d4 + v, s4 + v);
+      }
+      cp_async_commit();
+    };
+    int q = 0;                                   // chunks consumed
+#pragma unroll
+    for (int i = 0; i < C::NS - 1; ++i) stage(i);
+
     // ---- a1: point load (+ T^{-1}) ----
     if (tid < C::P) {
       int64_t idx = base + tid;
@@ -222,152 +231,220 @@ __global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm
     }
     __syncthreads();
 
-    float acc[C::PT][C::CT];
-    float fpart[C::PT];
+    // acc[j][h]: column j, point pair h; acc = sum_k X[k][point] M[k][column],
+    // the next panel of the stream as M.  All threads call it together.
+    float2 acc[C::TC][4];
+    auto product = [&]() {
 #pragma unroll
-    for (int i = 0; i < C::PT; ++i) fpart[i] = 0.0f;
+      for (int j = 0; j < C::TC; ++j)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) acc[j][h] = make_float2(0.f, 0.f);
+      const float *xk = X + pb;
+#pragma unroll 1
+      for (int kc = 0; kc < C::NCHUNK; ++kc, ++q) {
+        cp_async_wait<C::NS - 2>();
+        __syncthreads();          // chunk q is there, chunk q - 1 and (kc = 0) X are done with
+        stage(q + C::NS - 1);
+        const float *mk = Ms + (q % C::NS) * C::KC * W + cb;
+#pragma unroll 4
+        for (int k = 0; k < C::KC; ++k, xk += C::XS, mk += W) {
+          const float4 xa = *reinterpret_cast<const float4 *>(xk);
+          const float4 xb = *reinterpret_cast<const float4 *>(xk + 16);
+          float4 wv[C::TC / 4];
+          wv[0] = *reinterpret_cast<const float4 *>(mk);
+          if (C::TC == 8) wv[C::TC / 4 - 1] = *reinterpret_cast<const float4 *>(mk + 32);
+#pragma unroll
+          for (int j = 0; j < C::TC; ++j) {
+            const float2 w = f2_splat(el4(wv[j / 4], j % 4));
+            acc[j][0] = f2_fma(make_float2(xa.x, xa.y), w, acc[j][0]);
+            acc[j][1] = f2_fma(make_float2(xa.z, xa.w), w, acc[j][1]);
+            acc[j][2] = f2_fma(make_float2(xb.x, xb.y), w, acc[j][2]);
+            acc[j][3] = f2_fma(make_float2(xb.z, xb.w), w, acc[j][3]);
+          }
+        }
+      }
+      __syncthreads();            // every warp has read X: it may be replaced
+    };
+    auto store_x = [&](int c, const float (&v)[8]) {
+      float *o = X + c * C::XS + pb;
+      *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<float4 *>(o + 16) = make_float4(v[4], v[5], v[6], v[7]);
+    };
 
     const int m = FF ? prm.ff : 0;
-    if (m > 0) {
+    if (FF) {
       // ---- Fourier features gamma(p) (2m = W values) as L0's input tile ----
-      // (columns not unrolled: this phase must not raise the kernel's registers)
+      // (not unrolled: this phase must not raise the kernel's registers)
 #pragma unroll 1
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
+      for (int j = 0; j < C::TC; ++j) {
+        const int c = column(j);
         const int fi = c < m ? c : c - m;
         const float bx = ffB[fi * 3 + 0], by = ffB[fi * 3 + 1], bz = ffB[fi * 3 + 2];
-#pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          const int pr = g * C::PT + i;
+#pragma unroll 1
+        for (int i = 0; i < C::TP; ++i) {
+          const int pr = point(i);
           const float4 p = Ps[pr];
           float sn, cs;
           ff_sincos(bx, by, bz, p.x, p.y, p.z, sn, cs);
-          X[pr * W + c] = c < m ? sn : cs;
+          X[c * C::XS + pr] = c < m ? sn : cs;
         }
       }
-      __syncthreads();
-      panel_product<W, PT_>(X, ff0_t, Ms, g, colbase, acc);
+      product();
     } else {
       // ---- a2: L0 (K = 3) on CUDA cores ----
 #pragma unroll
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
+      for (int j = 0; j < C::TC; ++j) {
+        const int c = column(j);
         const float w0x = w0[c * 3 + 0], w0y = w0[c * 3 + 1], w0z = w0[c * 3 + 2];
 #pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          float4 p = Ps[g * C::PT + i];
-          acc[i][j] = fmaf(w0x, p.x, fmaf(w0y, p.y, w0z * p.z));
+        for (int h = 0; h < 4; ++h) {
+          const float4 p = Ps[point(2 * h)], r = Ps[point(2 * h + 1)];
+          acc[j][h] = make_float2(fmaf(w0x, p.x, fmaf(w0y, p.y, w0z * p.z)),
+                                  fmaf(w0x, r.x, fmaf(w0y, r.y, w0z * r.z)));
         }
       }
     }
 
     // ---- a3/a4/a5: hidden layers, activation epilogue, output unit ----
-    for (int l = 0; l < L; ++l) {
-      if (l > 0) {
-        float *t = X; X = Y; Y = t;
-        panel_product<W, PT_>(X, fwd_t + (size_t)(l - 1) * W * W, Ms, g, colbase, acc);
+    // (the last layer, like the last reverse product below, stands outside its
+    // loop, so that the sums over columns take no registers inside it)
+    auto activate = [&](int j, float bc, float (&h)[8], float (&s)[8]) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float z = (i & 1 ? acc[j][i / 2].y : acc[j][i / 2].x) + bc;
+        act_and_slope(z, beta, inv_beta, prm.relu, h[i], s[i]);
       }
+    };
+#pragma unroll 1
+    for (int l = 0; l < L - 1; ++l) {
+      if (l > 0) product();
       const float *b = bias + (size_t)l * W;
-      const bool last = (l == L - 1);
       const bool feeds_skip = (skip > 0 && l == skip - 1);
 #pragma unroll
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
-        const float bc = b[c];
-        const float wo = last ? wout[c] : 0.0f;
+      for (int j = 0; j < C::TC; ++j) {
+        const int c = column(j);
+        float h[8], s[8];
+        activate(j, b[c], h, s);
+        *slot(l, j, 0) = make_float4(s[0], s[1], s[2], s[3]);
+        *slot(l, j, 1) = make_float4(s[4], s[5], s[6], s[7]);
+        if (feeds_skip) {
 #pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          float h, s;
-          act_and_slope(acc[i][j] + bc, beta, inv_beta, prm.relu, h, s);
-          const int pr = g * C::PT + i;
-          if (last) {
-            fpart[i] = fmaf(wo, h, fpart[i]);
-            Y[pr * W + c] = s * wo;          // delta_{L-1} = sigmoid' * w_out
-          } else {
-            *slot(l, i, j) = s;
-            float v = h;
-            if (feeds_skip) {
-              if (c < nshort) {
-                v = h * kInvSqrt2;
-              } else {
-                float4 p = Ps[pr];
-                const int k = c - nshort;
-                v = (k == 0 ? p.x : k == 1 ? p.y : p.z) * kInvSqrt2;
-              }
+          for (int i = 0; i < 8; ++i) {
+            float v = h[i];
+            if (c >= nshort) {
+              const float4 p = Ps[point(i)];
+              const int k = c - nshort;
+              v = k == 0 ? p.x : k == 1 ? p.y : p.z;
             }
-            Y[pr * W + c] = v;
+            h[i] = v * kInvSqrt2;
           }
         }
+        store_x(c, h);
       }
-      __syncthreads();
+    }
+    if (L > 1) product();
+    float fpart[C::TP];
+#pragma unroll
+    for (int i = 0; i < C::TP; ++i) fpart[i] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < C::TC; ++j) {
+      const int c = column(j);
+      const float wo = wout[c];
+      float h[8], s[8];
+      activate(j, bias[(size_t)(L - 1) * W + c], h, s);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        fpart[i] = fmaf(wo, h[i], fpart[i]);
+        h[i] = s[i] * wo;                    // delta_{L-1} = sigmoid' * w_out
+      }
+      store_x(c, h);
     }
 
-    // f: reduce the partial dot products over lanes, then over the WG warps
+    // f: reduce the partial dot products over the warp's columns
 #pragma unroll
-    for (int i = 0; i < C::PT; ++i) {
+    for (int i = 0; i < C::TP; ++i) {
       float v = fpart[i];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[(part * C::P + g * C::PT + i) * 4 + 3] = v;
+      for (int o = 1; o < 32; o <<= 2) v += __shfl_xor_sync(0xffffffffu, v, o);   // the bits of lc
+      if (lc == 0) red[(cw * C::P + point(i)) * 4 + 3] = v;
     }
 
     // ---- a6: Jacobian-transpose chain ----
-    float gp[C::PT][3];
+    // d = delta_{l-1} of column j, from the product W_l^T delta_l in acc
+    auto reverse_delta = [&](int l, int j, float (&d)[8]) {
+      const int c = column(j);
+      const float4 s0 = *slot(l - 1, j, 0), s1 = *slot(l - 1, j, 1);
 #pragma unroll
-    for (int i = 0; i < C::PT; ++i) gp[i][0] = gp[i][1] = gp[i][2] = 0.0f;
-    for (int l = L - 1; l >= 1; --l) {
-      float *t = X; X = Y; Y = t;                       // X = delta_l
-      panel_product<W, PT_>(X, bwdw + (size_t)(l - 1) * W * W, Ms, g, colbase, acc);
-      const bool at_skip = (skip > 0 && l == skip);
-#pragma unroll
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
-#pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          const int pr = g * C::PT + i;
-          float u = acc[i][j];
-          if (at_skip) {
-            u *= kInvSqrt2;
-            if (c >= nshort) {                 // direct path to the input
-              dir[pr * 4 + (c - nshort)] += u;
-              u = 0.0f;
-            }
-          }
-          const float d = *slot(l - 1, i, j) * u;
-          if (l - 1 > 0 || m > 0) {
-            Y[pr * W + c] = d;                 // delta_{l-1} (delta_0 feeds W_0^T below)
-          } else {
-            gp[i][0] = fmaf(d, w0[c * 3 + 0], gp[i][0]);
-            gp[i][1] = fmaf(d, w0[c * 3 + 1], gp[i][1]);
-            gp[i][2] = fmaf(d, w0[c * 3 + 2], gp[i][2]);
+      for (int i = 0; i < 8; ++i) {
+        float u = i & 1 ? acc[j][i / 2].y : acc[j][i / 2].x;
+        if (skip > 0 && l == skip) {
+          u *= kInvSqrt2;
+          if (c >= nshort) {                 // direct path to the input
+            dir[point(i) * 4 + (c - nshort)] += u;
+            u = 0.0f;
           }
         }
+        d[i] = el4(i < 4 ? s0 : s1, i & 3) * u;
       }
-      __syncthreads();
+    };
+#pragma unroll 1
+    for (int l = L - 1; l >= (FF ? 1 : 2); --l) {
+      product();
+#pragma unroll
+      for (int j = 0; j < C::TC; ++j) {
+        float d[8];
+        reverse_delta(l, j, d);
+        store_x(column(j), d);
+      }
     }
-    if (m > 0) {
-      // ---- g_gamma = W_0^T delta_0, then through the feature Jacobian ----
+    if (FF || L > 1) product();              // W_1^T delta_1, or g_gamma = W_0^T delta_0
+    float gp[C::TP][3];
+#pragma unroll
+    for (int i = 0; i < C::TP; ++i) gp[i][0] = gp[i][1] = gp[i][2] = 0.0f;
+    if (!FF) {
+      // grad f += delta_0 W_0 (L = 1: delta_0 = sigmoid'(z_0) * w_out sits in X)
+#pragma unroll
+      for (int j = 0; j < C::TC; ++j) {
+        const int c = column(j);
+        float d[8];
+        if (L > 1) {
+          reverse_delta(1, j, d);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) d[i] = X[c * C::XS + point(i)];
+        }
+        const float wx = w0[c * 3 + 0], wy = w0[c * 3 + 1], wz = w0[c * 3 + 2];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          gp[i][0] = fmaf(d[i], wx, gp[i][0]);
+          gp[i][1] = fmaf(d[i], wy, gp[i][1]);
+          gp[i][2] = fmaf(d[i], wz, gp[i][2]);
+        }
+      }
+    }
+    if (FF) {
+      // ---- g_gamma through the feature Jacobian ----
       //   d sin(2 pi b.p)/dp = 2 pi cos(2 pi b.p) b,
       //   d cos(2 pi b.p)/dp = -2 pi sin(2 pi b.p) b
-      float *t = X; X = Y; Y = t;                       // X = delta_0
-      panel_product<W, PT_>(X, ff0, Ms, g, colbase, acc);
-      // park g_gamma in Y (each thread its own elements, so no barrier), so
+      // park g_gamma in X (each thread its own elements, so no barrier), so
       // that acc is dead while the sines and cosines are evaluated
 #pragma unroll
-      for (int j = 0; j < C::CT; ++j)
-#pragma unroll
-        for (int i = 0; i < C::PT; ++i) Y[(g * C::PT + i) * W + colbase + 32 * j] = acc[i][j];
+      for (int j = 0; j < C::TC; ++j) {
+        const float g[8] = {acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y,
+                            acc[j][2].x, acc[j][2].y, acc[j][3].x, acc[j][3].y};
+        store_x(column(j), g);
+      }
       constexpr float kTwoPi = 6.28318530717958648f;
 #pragma unroll 1
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
+      for (int j = 0; j < C::TC; ++j) {
+        const int c = column(j);
         const int fi = c < m ? c : c - m;
         const float bx = ffB[fi * 3 + 0], by = ffB[fi * 3 + 1], bz = ffB[fi * 3 + 2];
 #pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          const int pr = g * C::PT + i;
+        for (int i = 0; i < C::TP; ++i) {
+          const int pr = point(i);
           const float4 p = Ps[pr];
-          const float gg = Y[pr * W + c];
+          const float gg = X[c * C::XS + pr];
           float sn, cs;
           ff_sincos(bx, by, bz, p.x, p.y, p.z, sn, cs);
           const float coef = kTwoPi * (c < m ? gg * cs : -gg * sn);
@@ -376,28 +453,15 @@ __global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm
           gp[i][2] = fmaf(coef, bz, gp[i][2]);
         }
       }
-    } else if (L == 1) {
-      // no hidden-to-hidden product: delta_0 = sigmoid'(z_0) * w_out sits in Y
-#pragma unroll
-      for (int j = 0; j < C::CT; ++j) {
-        const int c = colbase + 32 * j;
-#pragma unroll
-        for (int i = 0; i < C::PT; ++i) {
-          const float d = Y[(g * C::PT + i) * W + c];
-          gp[i][0] = fmaf(d, w0[c * 3 + 0], gp[i][0]);
-          gp[i][1] = fmaf(d, w0[c * 3 + 1], gp[i][1]);
-          gp[i][2] = fmaf(d, w0[c * 3 + 2], gp[i][2]);
-        }
-      }
     }
 #pragma unroll
-    for (int i = 0; i < C::PT; ++i) {
+    for (int i = 0; i < C::TP; ++i) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         float v = gp[i][k];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[(part * C::P + g * C::PT + i) * 4 + k] = v;
+        for (int o = 1; o < 32; o <<= 2) v += __shfl_xor_sync(0xffffffffu, v, o);   // the bits of lc
+        if (lc == 0) red[(cw * C::P + point(i)) * 4 + k] = v;
       }
     }
     __syncthreads();
@@ -408,8 +472,8 @@ __global__ void __launch_bounds__(kThreads, 1) query_fp32_kernel(QueryParams prm
       float gx = dir[tid * 4 + 0], gy = dir[tid * 4 + 1], gz = dir[tid * 4 + 2];
       float f = bout[0];
 #pragma unroll
-      for (int q = 0; q < C::WG; ++q) {
-        const float *r = red + (q * C::P + tid) * 4;
+      for (int w = 0; w < C::CW; ++w) {
+        const float *r = red + (w * C::P + tid) * 4;
         gx += r[0]; gy += r[1]; gz += r[2]; f += r[3];
       }
       if (tid < nvalid) {
@@ -455,7 +519,7 @@ int per_sm_t() {
   // known once its opt-in attribute is set
   cudaFuncSetAttribute(query_fp32_kernel<W, PT_, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)C::SMEM_BYTES);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, query_fp32_kernel<W, PT_, FF>, kThreads,
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, query_fp32_kernel<W, PT_, FF>, C::THREADS,
                                                 C::SMEM_BYTES);
   return per_sm < 1 ? 1 : per_sm;
 }
@@ -467,7 +531,7 @@ cudaError_t launch_t(const QueryParams &p, int grid, cudaStream_t s) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  query_fp32_kernel<W, PT_, FF><<<grid, kThreads, C::SMEM_BYTES, s>>>(p);
+  query_fp32_kernel<W, PT_, FF><<<grid, C::THREADS, C::SMEM_BYTES, s>>>(p);
   return cudaGetLastError();
 }
 
