@@ -8,8 +8,8 @@
 //   dL/dW_l = (1/n) sum_i a_i delta_l(i) x_l(i)^T,   dL/db_l = (1/n) sum_i a_i delta_l(i),
 // x_l the layer's input.  The training form of the tensor-core kernel writes
 // every layer's A operand out (h_l on the forward pass, delta_l on the
-// reverse pass, 16-bit, one row per point); the rows of delta are then
-// multiplied by a_i (a sign flip or a zero: exact in 16 bits), the
+// reverse pass, 16-bit, one row per point); one pass multiplies the rows of
+// delta by a_i (a sign flip or a zero: exact in 16 bits) and sums them, the
 // hidden-layer weight gradients are contractions over the points on the
 // tensor cores (wgrad_tc.cu: tcgen05, FP32 accumulation in TMEM, split over
 // the points and reduced in a fixed order), and the remaining sums (biases, W_0 on p, the skip layer's
@@ -69,34 +69,19 @@ __global__ void l1_sign_kernel(const float4 *__restrict__ ns, const float *__res
   }
 }
 
-__global__ void l1_loss_kernel(const float *__restrict__ loss_part, int nb, int64_t n,
-                               float *__restrict__ loss) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// One block: thread t sums parts t, t + 256, .. in FP64, then a tree in a fixed
+// order (one thread over the 977 parts of 250,000 points took 80 us).
+__global__ void __launch_bounds__(256) l1_loss_kernel(const float *__restrict__ loss_part, int nb,
+                                                      int64_t n, float *__restrict__ loss) {
+  __shared__ double red[256];
   double t = 0.0;
-  for (int b = 0; b < nb; ++b) t += loss_part[b];
-  *loss = (float)(t / (double)n);
-}
-
-// delta rows times a_i: flip the sign bit of every 16-bit value, or zero it
-// (16 bytes = 8 values per access).
-__global__ void scale_rows_kernel(uint4 *__restrict__ d, int64_t vecs, int64_t n_pad, int W,
-                                  const float *__restrict__ a) {
-  const int64_t per_row = W / 8;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < vecs;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const float s = a[(t / per_row) % n_pad];
-    if (s > 0.f) continue;
-    uint4 v = d[t];
-    if (s == 0.f) {
-      v = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-      v.x ^= 0x80008000u;
-      v.y ^= 0x80008000u;
-      v.z ^= 0x80008000u;
-      v.w ^= 0x80008000u;
-    }
-    d[t] = v;
+  for (int b = threadIdx.x; b < nb; b += 256) t += loss_part[b];
+  red[threadIdx.x] = t;
+  for (int o = 128; o > 0; o >>= 1) {
+    __syncthreads();
+    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
   }
+  if (threadIdx.x == 0) *loss = (float)(red[0] / (double)n);
 }
 
 __device__ __forceinline__ float2 unpack16(uint32_t w, int fp16) {
@@ -104,118 +89,164 @@ __device__ __forceinline__ float2 unpack16(uint32_t w, int fp16) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w));
 }
 
-// Per-block partial sums over kRowsPerBlock points, for job j = blockIdx.y:
-//   j <  L : sum_i delta_j(i)[c]                         (bias of layer j)
-//   j == L : sum_i delta_0(i)[c] p_i[k], k = 0..2         (W_0; not for ff)
-//   j == L+1: sum_i delta_s(i)[c] p_i[k] / sqrt(2)        (skip layer s, its p columns)
-//   j == L+2: sum_i a_i h_{L-1}(i)[c]; and sum_i a_i      (w_out, b_out)
-// Thread t covers columns 8t .. 8t+7 (one 16-byte load per row); part[j][block][c][3].
-__global__ void small_partials_kernel(const uint16_t *__restrict__ save_h,
-                                      const uint16_t *__restrict__ save_d,
-                                      const float4 *__restrict__ pts, const float *__restrict__ a,
-                                      int L, int W, int skip, int ff, int64_t n, int64_t n_pad,
-                                      int fp16, float *__restrict__ part) {
+// One pass over the saved deltas: rows times a_i in place (a sign flip or a
+// zero; rows with a_i > 0 are not written) and, of the scaled rows, partial sums
+// over kRowsPerBlock points.  blockIdx.y = j < L is layer j, which gives
+//   part[j]  : sum_i delta_j(i)[c]                        (its bias),
+//   part[L]  : sum_i delta_0(i)[c] p_i[k], k = 0..2        (j = 0: W_0; not for ff),
+//   part[L+1]: sum_i delta_s(i)[c] p_i[k] / sqrt(2)        (j = s: the skip layer's p columns);
+// j = L gives part[L+2]: sum_i a_i h_{L-1}(i)[c], and sum_i a_i (w_out, b_out).
+// Thread t covers columns 8t .. 8t+7 (one 16-byte load per row), four rows in
+// flight; the sums run in row order; part[job][block][c][3].
+// Bound: memory, one read of every saved delta and one write of about half of
+// them.  As two passes (scale, then sum, the sums reading layer 0 and the skip
+// layer once more) they took 0.39 + 0.47 ms for 250,000 points of 3-512x8-1;
+// together 0.565 ms (5.9 TB/s).
+template <bool kP>      // with the sums over p
+__device__ __forceinline__ void scale_and_sum(uint16_t *__restrict__ d, const float4 *__restrict__ pts,
+                                              const float *__restrict__ a, float sc, int64_t r0,
+                                              int64_t r1, int64_t n, int W, int c, int fp16,
+                                              float (&sum)[8], float (&psum)[8][3]) {
+  for (int64_t r4 = r0; r4 < r1; r4 += 4) {         // r1 - r0 is a multiple of 128
+    uint4 wq[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) wq[i] = *reinterpret_cast<const uint4 *>(d + (size_t)(r4 + i) * W + c);
+    const float4 a4 = *reinterpret_cast<const float4 *>(a + r4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float s = i == 0 ? a4.x : i == 1 ? a4.y : i == 2 ? a4.z : a4.w;
+      if (!(s > 0.f)) {
+        const uint32_t keep = s == 0.f ? 0u : ~0u, flip = s == 0.f ? 0u : 0x80008000u;
+        wq[i] = make_uint4((wq[i].x & keep) ^ flip, (wq[i].y & keep) ^ flip, (wq[i].z & keep) ^ flip,
+                           (wq[i].w & keep) ^ flip);
+        *reinterpret_cast<uint4 *>(d + (size_t)(r4 + i) * W + c) = wq[i];
+      }
+      const uint32_t ww[4] = {wq[i].x, wq[i].y, wq[i].z, wq[i].w};
+      float q[3];
+      if (kP) {
+        const int64_t r = r4 + i;
+        const float4 p = r < n ? pts[r] : make_float4(0.f, 0.f, 0.f, 0.f);
+        q[0] = p.x * sc; q[1] = p.y * sc; q[2] = p.z * sc;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float2 f2 = unpack16(ww[u / 2], fp16);
+        const float v = u & 1 ? f2.y : f2.x;
+        sum[u] += v;
+        if (kP) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) psum[u][k] = fmaf(v, q[k], psum[u][k]);
+        }
+      }
+    }
+  }
+}
+
+__global__ void scale_sums_kernel(const uint16_t *__restrict__ save_h, uint16_t *__restrict__ save_d,
+                                  const float4 *__restrict__ pts, const float *__restrict__ a, int L,
+                                  int W, int skip, int ff, int64_t n, int64_t n_pad, int fp16,
+                                  float *__restrict__ part) {
   const int j = blockIdx.y;
   const int c = 8 * threadIdx.x;
   if (c >= W) return;
   const int64_t r0 = (int64_t)blockIdx.x * kRowsPerBlock;
   int64_t r1 = r0 + kRowsPerBlock;
   if (r1 > n_pad) r1 = n_pad;
-  const uint16_t *src = nullptr;
-  if (j < L) src = save_d + (size_t)j * n_pad * W;
-  else if (j == L) src = ff ? nullptr : save_d;
-  else if (j == L + 1) src = skip > 0 ? save_d + (size_t)skip * n_pad * W : nullptr;
-  else src = save_h + (size_t)(L - 1) * n_pad * W;
-  float acc[8][3];
+  float sum[8], psum[8][3], asum = 0.f;
 #pragma unroll
-  for (int u = 0; u < 8; ++u) acc[u][0] = acc[u][1] = acc[u][2] = 0.f;
-  float asum = 0.f;
-  if (src) {
-    // four rows' loads in flight per thread (r1 - r0 is a multiple of 128;
-    // four measured faster than one or eight);
-    // the sums still run in row order
+  for (int u = 0; u < 8; ++u) sum[u] = psum[u][0] = psum[u][1] = psum[u][2] = 0.f;
+  auto out = [&](int job) { return part + (((size_t)job * gridDim.x + blockIdx.x) * W + c) * 3; };
+  if (j < L) {
+    uint16_t *d = save_d + (size_t)j * n_pad * W;
+    const bool first = j == 0 && !ff, at_skip = skip > 0 && j == skip;
+    if (first || at_skip) {
+      scale_and_sum<true>(d, pts, a, first ? 1.f : kInvSqrt2, r0, r1, n, W, c, fp16, sum, psum);
+      float *o = out(first ? L : L + 1);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o[3 * u + k] = psum[u][k];
+    } else {
+      scale_and_sum<false>(d, pts, a, 0.f, r0, r1, n, W, c, fp16, sum, psum);
+    }
+  } else {
+    const uint16_t *h = save_h + (size_t)(L - 1) * n_pad * W;
     for (int64_t r4 = r0; r4 < r1; r4 += 4) {
       uint4 wq[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) wq[i] = *reinterpret_cast<const uint4 *>(src + (size_t)(r4 + i) * W + c);
+      for (int i = 0; i < 4; ++i) wq[i] = *reinterpret_cast<const uint4 *>(h + (size_t)(r4 + i) * W + c);
+      const float4 a4 = *reinterpret_cast<const float4 *>(a + r4);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int64_t r = r4 + i;
+        const float s = i == 0 ? a4.x : i == 1 ? a4.y : i == 2 ? a4.z : a4.w;
         const uint32_t ww[4] = {wq[i].x, wq[i].y, wq[i].z, wq[i].w};
-        float v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float2 f2 = unpack16(ww[u], fp16);
-          v[2 * u] = f2.x;
-          v[2 * u + 1] = f2.y;
+        for (int u = 0; u < 8; ++u) {
+          const float2 f2 = unpack16(ww[u / 2], fp16);
+          sum[u] = fmaf(s, u & 1 ? f2.y : f2.x, sum[u]);
         }
-        if (j < L) {
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u][0] += v[u];
-        } else if (j <= L + 1) {
-          float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (r < n) p = pts[r];
-          const float sc = j == L ? 1.f : kInvSqrt2;
-          const float q[3] = {p.x * sc, p.y * sc, p.z * sc};
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) acc[u][k] = fmaf(v[u], q[k], acc[u][k]);
-        } else {
-          const float s = a[r];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u][0] = fmaf(s, v[u], acc[u][0]);
-          asum += s;
-        }
+        asum += s;
       }
     }
   }
-  float *o = part + (((size_t)j * gridDim.x + blockIdx.x) * W + c) * 3;
+  float *o = out(j < L ? j : L + 2);
 #pragma unroll
-  for (int u = 0; u < 8; ++u)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) o[3 * u + k] = acc[u][k];
-  if (j == L + 2 && threadIdx.x == 0) o[2] = asum;   // column 0, slot 2: sum a_i
+  for (int u = 0; u < 8; ++u) {
+    o[3 * u] = sum[u];
+    o[3 * u + 1] = o[3 * u + 2] = 0.f;
+  }
+  if (j == L && threadIdx.x == 0) o[2] = asum;   // column 0, slot 2: sum a_i
 }
 
-// small[j][c][k] = sum over blocks, in block order.
-__global__ void small_reduce_kernel(const float *__restrict__ part, int jobs, int nb, int W,
-                                    float *__restrict__ small) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// small[j][c][k] = sum over blocks: 8 threads per element take every eighth
+// block each, then their sums are added in order.
+constexpr int kReduceWays = 8;
+__global__ void __launch_bounds__(32 * kReduceWays) small_reduce_kernel(const float *__restrict__ part,
+                                                                        int jobs, int nb, int W,
+                                                                        float *__restrict__ small) {
+  __shared__ float red[kReduceWays][32];
+  const int lane = threadIdx.x & 31, way = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * 32 + lane;     // jobs * 3 W is a multiple of 32
   const int64_t per_job = (int64_t)W * 3;
-  if (t >= (int64_t)jobs * per_job) return;
   const int j = (int)(t / per_job);
   const int64_t e = t % per_job;
   float s = 0.f;
-  for (int b = 0; b < nb; ++b) s += part[((size_t)j * nb + b) * per_job + e];
-  small[t] = s;
+  for (int b = way; b < nb; b += kReduceWays) s += part[((size_t)j * nb + b) * per_job + e];
+  red[way][lane] = s;
+  __syncthreads();
+  if (way == 0) {
+#pragma unroll
+    for (int w = 1; w < kReduceWays; ++w) s += red[w][lane];
+    small[t] = s;
+  }
 }
 
 // The gradient in blob layout, times 1/n.
+// Element t of the blob has a 32-bit index (at most 63 layers of 512 x 512), and
+// W is a power of two (256 or 512), wlog its logarithm.
 __global__ void scatter_grad_kernel(const float *__restrict__ G, const float *__restrict__ small,
-                                    BlobPlan plan, int64_t total, float inv_n,
+                                    BlobPlan plan, int total, int wlog, float inv_n,
                                     float *__restrict__ g) {
   const int L = plan.L, W = plan.W;
-  const int64_t per_job = (int64_t)W * 3;
-  auto sm = [&](int j, int c, int k) { return small[j * per_job + (int64_t)c * 3 + k]; };
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
+  const int per_job = W * 3;
+  auto sm = [&](int j, int c, int k) { return small[j * per_job + c * 3 + k]; };
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
     if (t < plan.woff[0]) {                       // the frequencies B: not trained
       g[t] = 0.f;
       continue;
     }
     int l = 0;
-    while (l < L && t >= plan.woff[l + 1]) ++l;   // layer of element t
+    while (l < L && t >= (int)plan.woff[l + 1]) ++l;   // layer of element t
     float v;
-    if (t >= plan.boff[l]) {                      // bias
-      const int nn = (int)(t - plan.boff[l]);
+    if (t >= (int)plan.boff[l]) {                 // bias
+      const int nn = t - (int)plan.boff[l];
       v = l < L ? sm(l, nn, 0) : sm(L + 2, 0, 2);
     } else {
-      const int64_t e = t - plan.woff[l];
+      const int e = t - (int)plan.woff[l];
+      const int nn = e >> wlog, k = e & (W - 1);
       if (plan.ff > 0 && l < L) {
         // G_l[n][c] for every layer; layer 0's columns are in the kernel's
         // feature order: feature k = s m + 64 g + i sits in column 128 g + 64 s + i
-        const int nn = (int)(e / W), k = (int)(e % W);
         int c = k;
         if (l == 0) {
           const int sgn = k / plan.ff, j = k % plan.ff;
@@ -223,11 +254,10 @@ __global__ void scatter_grad_kernel(const float *__restrict__ G, const float *__
         }
         v = G[((size_t)l * W + nn) * W + c];
       } else if (l == 0) {
-        v = sm(L, (int)(e / 3), (int)(e % 3));
+        v = sm(L, e / 3, e % 3);
       } else if (l == L) {
-        v = sm(L + 2, (int)e, 0);
+        v = sm(L + 2, e, 0);
       } else {
-        const int nn = (int)(e / W), k = (int)(e % W);
         v = (l == plan.skip && k >= W - 3) ? sm(L + 1, nn, k - (W - 3))
                                            : G[((size_t)(l - 1) * W + nn) * W + k];
       }
@@ -346,13 +376,12 @@ extern "C" nsdf_status nsdf_l1_grad(nsdf_ctx *ctx, const float *pts, int64_t n, 
   cudaError_t e = ff ? launch_query_tc16_ff(p, *net, fp16, num_sms, s)
                      : launch_query_tc16_net(p, *net, fp16, num_sms, s);
   if (e != cudaSuccess) return NSDF_ERR_CUDA;
-  // 2. a_i and the loss; delta rows times a_i
+  // 2. a_i and the loss; delta rows times a_i and the small partial sums
   const int lb = (int)((n_pad + 255) / 256);
   l1_sign_kernel<<<lb, 256, 0, s>>>(t->ns, targets, n, n_pad, t->a, t->loss_part);
-  l1_loss_kernel<<<1, 32, 0, s>>>(t->loss_part, lb, n, loss ? loss : t->loss_tmp);
-  const int64_t vecs = (int64_t)L * n_pad * W / 8;
-  scale_rows_kernel<<<8 * num_sms, 256, 0, s>>>(reinterpret_cast<uint4 *>(t->save_d), vecs, n_pad,
-                                                W, t->a);
+  l1_loss_kernel<<<1, 256, 0, s>>>(t->loss_part, lb, n, loss ? loss : t->loss_tmp);
+  scale_sums_kernel<<<dim3(nb, L + 1), W / 8, 0, s>>>(t->save_h, t->save_d, p.pts, t->a, L, W, p.skip,
+                                                     p.ff, n, n_pad, fp16 ? 1 : 0, t->part);
   // 3. hidden-layer weight gradients on the tensor cores:
   //    G_l[n][k] = sum_i delta_l(i)[n] h_{l-1}(i)[k]
   WgradJob job{};
@@ -378,11 +407,8 @@ extern "C" nsdf_status nsdf_l1_grad(nsdf_ctx *ctx, const float *pts, int64_t n, 
   job.num_sms = num_sms;
   if (job.layers > 0 && launch_wgrad_tc(job, s) != cudaSuccess) return NSDF_ERR_CUDA;
   // 4. the small sums, reduced in block order
-  small_partials_kernel<<<dim3(nb, jobs), W / 8, 0, s>>>(t->save_h, t->save_d, p.pts, t->a, L, W,
-                                                         p.skip, p.ff, n, n_pad, fp16 ? 1 : 0,
-                                                         t->part);
   const int64_t nsmall = (int64_t)jobs * W * 3;
-  small_reduce_kernel<<<(int)((nsmall + 255) / 256), 256, 0, s>>>(t->part, jobs, nb, W, t->small);
+  small_reduce_kernel<<<(int)(nsmall / 32), 32 * kReduceWays, 0, s>>>(t->part, jobs, nb, W, t->small);
   // 5. scatter into the blob layout
   BlobPlan plan{};
   plan.L = L;
@@ -391,7 +417,7 @@ extern "C" nsdf_status nsdf_l1_grad(nsdf_ctx *ctx, const float *pts, int64_t n, 
   plan.ff = p.ff;
   const int64_t total = ctx_blob_offsets(ctx, plan.woff, plan.boff, plan.out);
   plan.woff[L + 1] = total;
-  scatter_grad_kernel<<<4 * num_sms, 256, 0, s>>>(t->G, t->small, plan, total, 1.0f / (float)n,
-                                                  g_weights);
+  scatter_grad_kernel<<<8 * num_sms, 256, 0, s>>>(t->G, t->small, plan, (int)total,
+                                                  W == 512 ? 9 : 8, 1.0f / (float)n, g_weights);
   return cudaGetLastError() == cudaSuccess ? NSDF_OK : NSDF_ERR_CUDA;
 }
