@@ -7,24 +7,41 @@
 //   x_new = 2 x - x_prev + dt^2 (sum_j k (|d_j| - r_j) d_j/|d_j| + (0, -g, 0)).
 // Gathering per vertex needs no atomics; every spring is evaluated from both
 // ends, with equal and opposite results.  x_new overwrites x_prev in place
-// (each thread reads and writes only its own x_prev entry).  The step is
-// memory-bound: one float4 read of x_prev, one write, and x reads that hit
-// L1/L2 for the neighbours.
+// (each thread reads and writes only its own x_prev entry).
+//
+// Bound: instruction issue and memory alike (48 B per vertex, 50 MB at 1024 x
+// 1024: 7.4 us at 6.8 TB/s).  With an IEEE square root and division per spring
+// (about 60 instructions of 590 per vertex) the issue slots were 77% busy; the
+// reciprocal square root with one Newton step needs 14 and carries the same
+// FP32 rounding.  1024 x 1024: 20.5 -> 16.4 us with x and x_prev from DRAM, 12.4 us from L2; tiles of 32 x 8 vertices read
+// 1.3 rows per row written.  Evaluating each spring once, in strips that pass
+// the scalars on by shuffles, measured 15.5 us (and 22.5 with the IEEE forms):
+// the shuffles and the lower occupancy cost more than the springs.
 
 #include "nsdf_internal.h"
 
 namespace nsdf {
 namespace {
 
-__global__ void __launch_bounds__(256) cloth_step_kernel(const float4 *__restrict__ x,
-                                                         float4 *__restrict__ xprev, int nx, int ny,
-                                                         float hx, float hz, float k, float g,
-                                                         float dt) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;   // column (along x)
-  const int i = blockIdx.y;                              // row (along z)
+constexpr int kTileX = 32, kTileY = 8;
+
+// k (|d| - rest) / |d| = k (1 - rest / |d|), 0 for a spring of no length.
+__device__ __forceinline__ float spring(float dx, float dy, float dz, float rest, float k) {
+  const float d2 = dx * dx + dy * dy + dz * dz;
+  float r = rsqrtf(d2);
+  r = fmaf(0.5f * r, fmaf(-d2 * r, r, 1.0f), r);   // to FP32 rounding
+  return d2 > 0.f ? k * fmaf(-rest, r, 1.0f) : 0.f;
+}
+
+__global__ void __launch_bounds__(kTileX *kTileY) cloth_step_kernel(const float4 *__restrict__ x,
+                                                                    float4 *__restrict__ xprev,
+                                                                    int nx, int ny, float hx, float hz,
+                                                                    float k, float g, float dt) {
+  const int j = blockIdx.x * kTileX + threadIdx.x % kTileX;   // column (along x)
+  const int i = blockIdx.y * kTileY + threadIdx.x / kTileX;   // row (along z)
   if (j >= nx || i >= ny) return;
   const int64_t v = (int64_t)i * nx + j;
-  const float4 p = x[v];
+  const float4 p = x[v], pp = xprev[v];
   const float hd = sqrtf(hx * hx + hz * hz);
   float ax = 0.f, ay = -g, az = 0.f;
   const int di[8] = {0, 0, -1, 1, -1, -1, 1, 1};
@@ -36,11 +53,9 @@ __global__ void __launch_bounds__(256) cloth_step_kernel(const float4 *__restric
     const float rest = s < 2 ? hx : (s < 4 ? hz : hd);
     const float4 q = x[(int64_t)ii * nx + jj];
     const float dx = q.x - p.x, dy = q.y - p.y, dz = q.z - p.z;
-    const float len = sqrtf(dx * dx + dy * dy + dz * dz);
-    const float f = len > 0.f ? k * (len - rest) / len : 0.f;
+    const float f = spring(dx, dy, dz, rest, k);
     ax = fmaf(f, dx, ax); ay = fmaf(f, dy, ay); az = fmaf(f, dz, az);
   }
-  const float4 pp = xprev[v];
   const float dt2 = dt * dt;
   float4 o;
   o.x = 2.f * p.x - pp.x + dt2 * ax;
@@ -64,9 +79,10 @@ extern "C" nsdf_status nsdf_cloth_step(const float *x, float *x_prev_inout, int 
     return NSDF_ERR_MISALIGNED;
   if (!nsdf::device_memory(x) || !nsdf::device_memory(x_prev_inout)) return NSDF_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  dim3 grid((nx + 255) / 256, ny);
-  nsdf::cloth_step_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4 *>(x),
-                                               reinterpret_cast<float4 *>(x_prev_inout), nx, ny,
-                                               hx, hz, k_over_m, g, dt);
+  const dim3 grid((unsigned)((nx + nsdf::kTileX - 1) / nsdf::kTileX),
+                  (unsigned)((ny + nsdf::kTileY - 1) / nsdf::kTileY));
+  nsdf::cloth_step_kernel<<<grid, nsdf::kTileX * nsdf::kTileY, 0, s>>>(
+      reinterpret_cast<const float4 *>(x), reinterpret_cast<float4 *>(x_prev_inout), nx, ny, hx, hz,
+      k_over_m, g, dt);
   return cudaGetLastError() == cudaSuccess ? NSDF_OK : NSDF_ERR_CUDA;
 }
