@@ -35,6 +35,17 @@
 // reloading the weights only when its range crosses into another body.
 // Every mbarrier wait is bounded (QueryParams::wait_budget); on expiry the
 // kernel records kDevTimeout and returns.
+//
+// A single network with at most one tile per SM (the small calls, where the
+// chain of one tile is all there is to wait for) runs query_w64_small_kernel:
+// a tile per CTA, two warpgroups per tile with 32 columns each, FP32 arithmetic
+// in f32x2 pairs and the weights arriving while L0 is computed.  Sums over the
+// 64 columns stay one chain in column order, which the second warpgroup takes
+// over from the first, so both kernels give the same bits.  4,096 points of
+// 3-64x3-1: 17.2 -> 12.3 us a call.  On large calls (1,048,576 points, grouped
+// scenes) that form measured 0.90-1.02 of this one's speed, with one or two
+// warpgroups per tile: the epilogues' latency, not their FP32 instructions,
+// bounds them.
 
 #include <cudaTypedefs.h>
 
@@ -62,7 +73,7 @@ constexpr int kSmallFloats = kW * 3 + kMaxHidden * kW + kW + 4;
 struct Layout {
   int whi, wlo, a, a_stride, small, bars, slot, total;
 };
-__host__ __device__ inline Layout layout(int L, bool split) {
+__host__ __device__ inline Layout layout(int L, bool split, int tiles = kTilesPerCta) {
   Layout o{};
   const int nh = L - 1;
   o.whi = 0;
@@ -70,7 +81,7 @@ __host__ __device__ inline Layout layout(int L, bool split) {
   o.a = o.wlo + (split ? nh * kWBytes : 0);
   o.a = (o.a + 1023) & ~1023;
   o.a_stride = split ? 2 * kABytes : kABytes;       // A_hi (then A_lo) per tile
-  o.small = o.a + kTilesPerCta * o.a_stride;
+  o.small = o.a + tiles * o.a_stride;
   o.bars = o.small + kSmallFloats * 4;
   o.slot = o.bars + 8 * kTilesPerCta;
   o.total = o.slot + 16;
@@ -80,8 +91,8 @@ __host__ __device__ inline Layout layout(int L, bool split) {
 // layers 0 .. L-2 (32 columns of FP16 pairs each); the CTA allocates a power
 // of two of at least both tiles' columns.
 __host__ __device__ inline int tile_cols(int L) { return kW + (L - 1) * 32; }
-__host__ __device__ inline int cta_cols(int L) {
-  const int need = kTilesPerCta * tile_cols(L);
+__host__ __device__ inline int cta_cols(int L, int tiles = kTilesPerCta) {
+  const int need = tiles * tile_cols(L);
   int c = 32;
   while (c < need) c <<= 1;
   return c;
@@ -161,6 +172,71 @@ __device__ __forceinline__ void store_a(uint8_t *Ahi, uint8_t *Alo, int r, int c
   }
 }
 
+// One round of products into the accumulator d: layer l's forward (A W_l^T)
+// or reverse (A W_l) product, A_hi at a0 and A_lo at al, W_l's parts at w0, w1.
+template <bool kF16>
+__device__ __forceinline__ void issue_round(uint32_t d, uint32_t a0, uint32_t al, uint32_t w0,
+                                            uint32_t w1, bool reverse) {
+  constexpr bool kSplit = !kF16;
+  constexpr uint32_t idesc_f = idesc_f16(kF16, kM, kW);
+  constexpr uint32_t idesc_r = idesc_f | (1u << 16);      // B (W_l read as W_l^T) MN-major
+#pragma unroll
+  for (int ks = 0; ks < kW / 16; ++ks) {
+    if (!reverse) {
+      mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc(w0 + 32 * ks), idesc_f, ks > 0 ? 1u : 0u);
+      if constexpr (kSplit) {
+        mma_f16(d, sw128_desc(al + 32 * ks), sw128_desc(w0 + 32 * ks), idesc_f, 1u);
+        mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc(w1 + 32 * ks), idesc_f, 1u);
+      }
+    } else {
+      // K = the layer's outputs n: W_l rows, 16 rows = two 1024-byte groups
+      mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc_mn(w0 + 2048 * ks, 8192), idesc_r,
+              ks > 0 ? 1u : 0u);
+      if constexpr (kSplit) {
+        mma_f16(d, sw128_desc(al + 32 * ks), sw128_desc_mn(w0 + 2048 * ks, 8192), idesc_r, 1u);
+        mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc_mn(w1 + 2048 * ks, 8192), idesc_r, 1u);
+      }
+    }
+  }
+}
+
+// a . (x, y, z) with every rounding written out, so that both kernels give the
+// same bits.
+__device__ __forceinline__ float dot3(const float *a, float x, float y, float z) {
+  return fmaf(a[2], z, fmaf(a[0], x, a[1] * y));
+}
+// p' = T^{-1} p (rows 0..2 of the inverse, or null).
+__device__ __forceinline__ float3 to_body(const float *Ti, const float4 &p) {
+  if (!Ti) return make_float3(p.x, p.y, p.z);
+  return make_float3(dot3(Ti, p.x, p.y, p.z) + Ti[3], dot3(Ti + 4, p.x, p.y, p.z) + Ti[7],
+                     dot3(Ti + 8, p.x, p.y, p.z) + Ti[11]);
+}
+// Eq. 2, the test and Eq. 3 for point idx (position pw) from f and grad f.
+__device__ __forceinline__ void finish(const QueryParams &prm, int64_t idx, const float4 &pw, float f,
+                                       float gx, float gy, float gz, const float *R) {
+  const float nrm = sqrtf(fmaf(gz, gz, fmaf(gx, gx, gy * gy)));
+  float nx = 0.f, ny = 0.f, nz = 0.f;
+  if (nrm >= 1e-20f) { nx = gx / nrm; ny = gy / nrm; nz = gz / nrm; }
+  if (!prm.collide) {
+    if (prm.raw_gradient) { nx = gx; ny = gy; nz = gz; }
+    prm.out_n_sdf[idx] = make_float4(nx, ny, nz, f);
+    return;
+  }
+  if (R) {
+    const float wx = dot3(R, nx, ny, nz), wy = dot3(R + 3, nx, ny, nz), wz = dot3(R + 6, nx, ny, nz);
+    nx = wx; ny = wy; nz = wz;
+  }
+  const bool hit = f < prm.eps;
+  float4 p = pw;
+  if (hit) {
+    const float d = prm.eps - f;
+    p.x = fmaf(d, nx, p.x); p.y = fmaf(d, ny, p.y); p.z = fmaf(d, nz, p.z);
+  }
+  if (prm.out_pts) prm.out_pts[idx] = p;
+  if (prm.out_n_sdf) prm.out_n_sdf[idx] = make_float4(nx, ny, nz, f);
+  if (prm.out_hit) prm.out_hit[idx] = hit ? 1 : 0;
+}
+
 template <bool kF16>
 __global__ void __launch_bounds__(kThreads, 2)
     query_w64_kernel(const __grid_constant__ QueryParams prm) {
@@ -205,8 +281,6 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int64_t pairs = (tiles + 1) / 2;
   const int64_t p0 = pairs * blockIdx.x / gridDim.x, p1 = pairs * (blockIdx.x + 1) / gridDim.x;
   const float neg_bl2e = -prm.beta * 1.4426950408889634f, inv_beta = 1.0f / prm.beta;
-  const uint32_t idesc_f = idesc_f16(kF16, kM, kW);
-  const uint32_t idesc_r = idesc_f | (1u << 16);          // B (W_l read as W_l^T) MN-major
   uint32_t phase = 0;
   bool ok = true;
   int loaded = -1;
@@ -224,24 +298,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       const uint32_t w0 = sbase + lay.whi + (l - 1) * kWBytes;
       const uint32_t w1 = sbase + lay.wlo + (l - 1) * kWBytes;
       const uint32_t d = tmem + (uint32_t)(wg * tile_cols(L));
-#pragma unroll
-      for (int ks = 0; ks < kW / 16; ++ks) {
-        if (!reverse) {
-          mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc(w0 + 32 * ks), idesc_f, ks > 0 ? 1u : 0u);
-          if constexpr (kSplit) {
-            mma_f16(d, sw128_desc(al + 32 * ks), sw128_desc(w0 + 32 * ks), idesc_f, 1u);
-            mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc(w1 + 32 * ks), idesc_f, 1u);
-          }
-        } else {
-          // K = the layer's outputs n: W_l rows, 16 rows = two 1024-byte groups
-          mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc_mn(w0 + 2048 * ks, 8192), idesc_r,
-                  ks > 0 ? 1u : 0u);
-          if constexpr (kSplit) {
-            mma_f16(d, sw128_desc(al + 32 * ks), sw128_desc_mn(w0 + 2048 * ks, 8192), idesc_r, 1u);
-            mma_f16(d, sw128_desc(a0 + 32 * ks), sw128_desc_mn(w1 + 2048 * ks, 8192), idesc_r, 1u);
-          }
-        }
-      }
+      issue_round<kF16>(d, a0, al, w0, w1, reverse);
       if (round != prm.drop_load) mma_commit(bar);
     }
     ++round;
@@ -312,7 +369,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     float4 pw = make_float4(0.f, 0.f, 0.f, 0.f);
     if (valid) pw = prm.pts[idx];
-    float px = pw.x, py = pw.y, pz = pw.z;
     const float *Ti = nullptr, *R = nullptr;
     if (grouped && prm.g_T) {
       Ti = prm.g_T + (size_t)kBodyFloats * k;
@@ -321,11 +377,8 @@ __global__ void __launch_bounds__(kThreads, 2)
       Ti = prm.Ti;
       R = prm.R;
     }
-    if (Ti) {
-      px = Ti[0] * pw.x + Ti[1] * pw.y + Ti[2] * pw.z + Ti[3];
-      py = Ti[4] * pw.x + Ti[5] * pw.y + Ti[6] * pw.z + Ti[7];
-      pz = Ti[8] * pw.x + Ti[9] * pw.y + Ti[10] * pw.z + Ti[11];
-    }
+    const float3 pb = to_body(Ti, pw);
+    const float px = pb.x, py = pb.y, pz = pb.z;
 
     // ---- L0 on CUDA cores ----
 #pragma unroll 1
@@ -417,32 +470,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (!ok) continue;        // the barrier at the top of the loop ends both warpgroups
 
     // ---- Eq. 2, the test and Eq. 3 ----
-    if (valid) {
-      f += sBo[0];
-      const float nrm = sqrtf(gx * gx + gy * gy + gz * gz);
-      float nx = 0.f, ny = 0.f, nz = 0.f;
-      if (nrm >= 1e-20f) { nx = gx / nrm; ny = gy / nrm; nz = gz / nrm; }
-      if (!prm.collide) {
-        if (prm.raw_gradient) { nx = gx; ny = gy; nz = gz; }
-        prm.out_n_sdf[idx] = make_float4(nx, ny, nz, f);
-      } else {
-        if (R) {
-          const float wx = R[0] * nx + R[1] * ny + R[2] * nz;
-          const float wy = R[3] * nx + R[4] * ny + R[5] * nz;
-          const float wz = R[6] * nx + R[7] * ny + R[8] * nz;
-          nx = wx; ny = wy; nz = wz;
-        }
-        const bool hit = f < prm.eps;
-        float4 p = pw;
-        if (hit) {
-          const float d = prm.eps - f;
-          p.x = fmaf(d, nx, p.x); p.y = fmaf(d, ny, p.y); p.z = fmaf(d, nz, p.z);
-        }
-        if (prm.out_pts) prm.out_pts[idx] = p;
-        if (prm.out_n_sdf) prm.out_n_sdf[idx] = make_float4(nx, ny, nz, f);
-        if (prm.out_hit) prm.out_hit[idx] = hit ? 1 : 0;
-      }
-    }
+    if (valid) finish(prm, idx, pw, f + sBo[0], gx, gy, gz, R);
   }
   if (!ok && lane == 0) atomicExch(prm.err, kDevTimeout);
   // drain: every product of the warpgroup has completed before TMEM is freed
@@ -457,6 +485,262 @@ __global__ void __launch_bounds__(kThreads, 2)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(ncols));
   }
+}
+
+// ---- small calls: one tile per CTA, two warpgroups per tile ----
+
+// Store / load 8 32-bit columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+      : "memory");
+}
+__device__ __forceinline__ float2 pair(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+__device__ __forceinline__ float2 bits2(const uint32_t (&r)[32], int j) {
+  return make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+}
+
+// 32 values of a row (and, split, their residuals) at columns c0 .. c0 + 31.
+template <bool kF16, bool kSplit>
+__device__ __forceinline__ void store_a2(uint8_t *Ahi, uint8_t *Alo, int r, int c0,
+                                         const float2 (&v)[16]) {
+  uint32_t hw[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) hw[j] = pack16<kF16>(v[j].x, v[j].y);
+  store_a_chunk(Ahi, r, c0, hw);
+  if constexpr (kSplit) {
+    uint32_t lw[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float2 d = f2_add(v[j], make_float2(-from16<kF16>(hw[j], false), -from16<kF16>(hw[j], true)));
+      lw[j] = pack16<kF16>(d.x, d.y);
+    }
+    store_a_chunk(Alo, r, c0, lw);
+  }
+}
+
+// FP32 weights in shared memory: W_0 [3][64], biases [n_hidden][64], w_out
+// [64], b_out; then a float4 per point that the first half of the columns
+// leaves for the second.
+constexpr int kSmallKernelFloats = kSmallFloats + kM * 4;
+__host__ inline int small_kernel_smem(int L, bool split) {
+  const Layout o = layout(L, split, 1);
+  return o.small + kSmallKernelFloats * 4 + 8 + 16 + 1024;
+}
+
+template <bool kF16>
+__global__ void __launch_bounds__(256, 1)
+    query_w64_small_kernel(const __grid_constant__ QueryParams prm) {
+  constexpr bool kSplit = !kF16;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                              ~uintptr_t(1023));
+  const int L = prm.n_hidden, nh = L - 1;
+  const Layout lay = layout(L, kSplit, 1);
+  const int tid = threadIdx.x, half = tid >> 7, r = tid & 127, q = r >> 5, lane = tid & 31;
+  const int cb = 32 * half;                       // this thread's columns cb .. cb + 31
+  const uint32_t sbase = smem_u32(smem);
+  float *sm = reinterpret_cast<float *>(smem + lay.small);
+  float *sW0 = sm, *sB = sm + kW * 3, *sWo = sB + kMaxHidden * kW, *sBo = sWo + kW;
+  float4 *xch = reinterpret_cast<float4 *>(sm + kSmallFloats);
+  const uint32_t off_bar = lay.small + kSmallKernelFloats * 4, bar = sbase + off_bar;
+  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + off_bar + 8);
+  uint8_t *Ahi = smem + lay.a, *Alo = Ahi + kABytes;
+  const long long budget = prm.wait_budget;
+  volatile int no_abort = 0;
+
+  // everything the tile needs is asked for at once
+  const int64_t idx = (int64_t)blockIdx.x * kM + r;
+  const bool valid = idx < prm.n;
+  float4 pw = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (valid) pw = prm.pts[idx];
+  for (int e = tid; e < nh * kW * 8; e += 256) {
+    const int i = e / (kW * 8), n = (e / 8) % kW, j = e % 8;
+    const size_t src = ((size_t)i * kW + n) * kW + 8 * j;
+    const uint32_t dst = sbase + i * kWBytes + n * 128 + ((j ^ (n & 7)) * 16);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + lay.whi), "l"(prm.fwd16 + src));
+    if constexpr (kSplit)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + lay.wlo), "l"(prm.fwd16_lo + src));
+  }
+  asm volatile("cp.async.commit_group;\n");
+  for (int e = tid; e < kW * 3; e += 256) sW0[(e % 3) * kW + e / 3] = __ldg(prm.w0 + e);
+  for (int e = tid; e < L * kW; e += 256) sB[e] = __ldg(prm.bias + e);
+  for (int e = tid; e < kW; e += 256) sWo[e] = __ldg(prm.wout + e);
+  if (tid == 0) {
+    sBo[0] = __ldg(prm.bout);
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  const uint32_t ncols = (uint32_t)cta_cols(L, 1);
+  if (tid < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     sbase + off_bar + 8),
+                 "r"(ncols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t tb = tmem + ((uint32_t)(32 * q) << 16);
+  const float neg_bl2e = -prm.beta * 1.4426950408889634f, inv_beta = 1.0f / prm.beta;
+  uint32_t phase = 0;
+  int round = 0;
+
+  auto issue = [&](int l, bool reverse) {
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (tid == 0) {
+      issue_round<kF16>(tmem, smem_u32(Ahi), smem_u32(Alo), sbase + lay.whi + (l - 1) * kWBytes,
+                        sbase + lay.wlo + (l - 1) * kWBytes, reverse);
+      if (round != prm.drop_load) mma_commit(bar);
+    }
+    ++round;
+  };
+  auto done = [&]() -> bool {          // the same for every thread
+    const bool ok = __syncthreads_and(mbar_wait(bar, phase, budget, &no_abort) ? 1 : 0) != 0;
+    if (ok) phase ^= 1u;
+    tc_fence_after();
+    return ok;
+  };
+  // activations v, slopes parked at layer j's TMEM columns
+  auto park = [&](int j, const float2 (&s)[16]) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      uint32_t sw[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) sw[i] = pack16<true>(s[8 * b + i].x, s[8 * b + i].y);
+      tmem_st8(tb + kW + 32 * j + ((cb + 16 * b) >> 1), sw);
+    }
+  };
+
+  // ---- L0 on CUDA cores ----
+  {
+    const float3 p = to_body(prm.has_T ? prm.Ti : nullptr, pw);
+    const float2 px = f2_splat(p.x), py = f2_splat(p.y), pz = f2_splat(p.z);
+    float2 h[16], s[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int c = cb + 2 * j;
+      const float2 z = f2_fma(pair(sW0 + c), px,
+                              f2_fma(pair(sW0 + kW + c), py,
+                                     f2_fma(pair(sW0 + 2 * kW + c), pz, pair(sB + c))));
+      act_f32x2(z, neg_bl2e, inv_beta, h[j], s[j]);
+    }
+    store_a2<kF16, kSplit>(Ahi, Alo, r, cb, h);
+    park(0, s);
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");      // the 16-bit weights
+  tmem_wait_st();
+
+  bool ok = true;
+  float f = 0.f;
+  float2 keep[16];          // what the chains over the columns still need
+  // ---- hidden layers (forward) ----
+  for (int l = 1; ok && l < L; ++l) {
+    issue(l, false);
+    if (!(ok = done())) break;
+    uint32_t raw[32];
+    tmem_ld32_async(tb + cb, raw);
+    tmem_wait_ld(raw);
+    float2 s[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      act_f32x2(f2_add(bits2(raw, j), pair(sB + l * kW + cb + 2 * j)), neg_bl2e, inv_beta, keep[j], s[j]);
+    if (l < L - 1) {
+      store_a2<kF16, kSplit>(Ahi, Alo, r, cb, keep);
+      park(l, s);
+      tmem_wait_st();
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) s[j] = f2_mul(s[j], pair(sWo + cb + 2 * j));
+      store_a2<kF16, kSplit>(Ahi, Alo, r, cb, s);       // delta_{L-1}: the reverse chain's A
+    }
+  }
+  auto add_f = [&]() {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      f = fmaf(sWo[cb + 2 * j], keep[j].x, f);
+      f = fmaf(sWo[cb + 2 * j + 1], keep[j].y, f);
+    }
+  };
+  if (ok && half == 0) {
+    add_f();
+    xch[r].x = f;
+  }
+  // ---- Jacobian-transpose chain: layers L-1 .. 1 ----
+  for (int l = L - 1; ok && l >= 1; --l) {
+    issue(l, true);
+    if (l == L - 1 && half == 1) {      // the second half's part of f, beside the product
+      f = xch[r].x;
+      add_f();
+    }
+    if (!(ok = done())) break;
+    uint32_t raw[32], sl[16];
+    tmem_ld32_async(tb + cb, raw);
+    tmem_ld16_async(tb + kW + 32 * (l - 1) + (cb >> 1), sl);
+    tmem_wait_ld(raw);
+    tmem_wait_ld(sl);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      keep[j] = f2_mul(__half22float2(*reinterpret_cast<const __half2 *>(&sl[j])), bits2(raw, j));
+    if (l > 1) store_a2<kF16, kSplit>(Ahi, Alo, r, cb, keep);
+  }
+  if (ok) {
+    float gx = 0.f, gy = 0.f, gz = 0.f;
+    auto add_g = [&]() {                // grad f = W_0^T delta_0
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int c = cb + 2 * j;
+        gx = fmaf(keep[j].x, sW0[c], gx);
+        gy = fmaf(keep[j].x, sW0[kW + c], gy);
+        gz = fmaf(keep[j].x, sW0[2 * kW + c], gz);
+        gx = fmaf(keep[j].y, sW0[c + 1], gx);
+        gy = fmaf(keep[j].y, sW0[kW + c + 1], gy);
+        gz = fmaf(keep[j].y, sW0[2 * kW + c + 1], gz);
+      }
+    };
+    if (half == 0) {
+      add_g();
+      xch[r] = make_float4(gx, gy, gz, 0.f);
+    }
+    __syncthreads();
+    if (half == 1 && valid) {
+      const float4 g = xch[r];
+      gx = g.x; gy = g.y; gz = g.z;
+      add_g();
+      finish(prm, idx, pw, f + sBo[0], gx, gy, gz, prm.has_T ? prm.R : nullptr);
+    }
+  } else if (lane == 0) {
+    atomicExch(prm.err, kDevTimeout);
+  }
+  // drain, as in query_w64_kernel
+  if (tid == 0) mma_commit(bar);
+  if (!done() && lane == 0) atomicExch(prm.err, kDevTimeout);
+  tc_fence_before();
+  __syncthreads();
+  if (tid < 32) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(ncols));
+  }
+}
+
+template <bool kF16>
+cudaError_t launch_small_t(const QueryParams &p, int64_t tiles, cudaStream_t s) {
+  // more shared memory than one CTA needs is asked for where two CTAs' TMEM
+  // columns would not fit an SM (at most 4 fit: 128 columns and more each)
+  const int need = small_kernel_smem(p.n_hidden, !kF16);
+  const int fit = 512 / cta_cols(p.n_hidden, 1), cap = 233472 / (fit + 1) - 1024 + 16;
+  const int smem = need > cap ? need : cap;
+  if (smem > 232448) return cudaErrorInvalidConfiguration;
+  cudaError_t e = cudaFuncSetAttribute(query_w64_small_kernel<kF16>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  query_w64_small_kernel<kF16><<<(int)tiles, 256, smem, s>>>(p);
+  return cudaGetLastError();
 }
 
 // Dynamic shared memory of a launch: the layout, plus padding so that no
@@ -530,6 +814,11 @@ int query_w64_ctas_per_sm(int n_hidden, bool fp16) {
 cudaError_t launch_query_w64(const QueryParams &p, bool fp16, int num_sms, int ctas_per_sm,
                              cudaStream_t s) {
   if (!query_w64_supported(p.width, p.n_hidden, p.skip)) return cudaErrorInvalidValue;
+  // one network, a tile per SM at most: the small kernel.  With 157 tiles (5
+  // more than SMs) both take 18.5 us, with 391 it is 6-14% slower.
+  const int64_t tiles = (p.n + kM - 1) / kM;
+  if (p.g_nets == 0 && tiles <= num_sms)
+    return fp16 ? launch_small_t<true>(p, tiles, s) : launch_small_t<false>(p, tiles, s);
   return fp16 ? launch_t<true>(p, num_sms, ctas_per_sm, s) : launch_t<false>(p, num_sms, ctas_per_sm, s);
 }
 
