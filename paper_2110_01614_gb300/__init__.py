@@ -109,8 +109,15 @@ def _work_list(pts, offsets, counts, max_total, out_pts, out_n_sdf, T=None):
 _HIT = (torch.uint8, torch.bool)
 
 
+# PyTorch's current stream as a raw handle: the call that torch.cuda.current_stream
+# wraps in a Stream object, without making one (0.3 us instead of 3.7 us a call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
