@@ -12,15 +12,19 @@
 // CTA's totals in shared memory.  Per k step a thread reads 16 bytes of weights
 // and 32 bytes of pairs for 16 paired FMAs.
 //
-// Layouts in shared memory: weights [n][k] with rows of 68 floats, serving the
-// forward product (four consecutive k of a row) and the reverse one (four
-// consecutive k of row c) alike; pairs [column][point] with rows of 132 floats,
-// so that eight neighbouring rows, and eight neighbouring point pairs, lie in
-// different banks.
+// Layouts in shared memory: weights [n][k] with the 16-byte chunk k / 4 of row n
+// at chunk (k / 4) ^ (n / 4 mod 8), so that the forward product (one chunk of
+// eight threads' rows) and the reverse one (eight chunks of a row) both read
+// eight different banks; pairs [column][point] with rows of 132 floats, so that
+// neighbouring rows lie in different banks.  Lanes that differ in bit 1 share
+// their columns, lanes that differ in bit 0 their points: 16-byte shared loads
+// then merge into two wavefronts instead of four.
 //
-// Bound: the FP32 pipe (50 K FMA a point with both streams).  Measured, one
-// call on 250,000 points with weight gradients (3-64-64-64-1): see the rule in
-// launch_backward.
+// Bound: the FP32 pipe (50 K FMA a point with both streams: 0.33 ms for 250,000
+// points at its rate).  Measured, 250,000 points of 3-64-64-64-1 with weight
+// gradients: general kernel 3.4 ms, this one 0.62 ms (0.64 with eight point pairs
+// and four columns per warp, whose shared loads take ten wavefronts a k step
+// where this mapping takes six).
 
 #include "backward.cuh"
 #include "f32x2.cuh"
@@ -31,7 +35,6 @@ namespace {
 constexpr int kW = 64;
 constexpr int kP = 64;                    // points per tile
 constexpr int kThreads = 256;
-constexpr int kWRow = kW + 4;             // floats per weight row
 constexpr int kARow = 2 * kP + 4;         // floats per row of pairs
 constexpr int kShort = kW - 3;            // outputs of the layer feeding a skip
 constexpr float kInvSqrt2 = 0.70710678118654752f;
@@ -39,8 +42,8 @@ constexpr float kInvSqrt2 = 0.70710678118654752f;
 // Shared-memory map, in floats.
 template <int L>
 struct Map {
-  static constexpr int w = 0;                              // [L-1][kW][kWRow]
-  static constexpr int a = w + (L - 1) * kW * kWRow;       // [L-1][kW][kARow]: layer inputs
+  static constexpr int w = 0;                              // [L-1][kW][kW], swizzled
+  static constexpr int a = w + (L - 1) * kW * kW;       // [L-1][kW][kARow]: layer inputs
   static constexpr int zb = a + (L - 1) * kW * kARow;      // [kW][kARow]
   static constexpr int gw = zb + kW * kARow;               // [L-1][4][kThreads] float4
   static constexpr int pv = gw + (L - 1) * 16 * kThreads;  // [3][kARow]: pairs (p, v)
@@ -63,6 +66,8 @@ __device__ __forceinline__ void softplus_and_slope(float z, float beta, float in
   s = (z >= 0.0f) ? inv : u * inv;
 }
 
+// Float offset of 16-byte chunk q of weight row n (rows of all layers in turn).
+__device__ __forceinline__ int swizzled(int n, int q) { return n * kW + ((q ^ ((n >> 2) & 7)) << 2); }
 __device__ __forceinline__ float2 lo(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi(const float4 &v) { return make_float2(v.z, v.w); }
 __device__ __forceinline__ float el(const float4 &v, int i) {
@@ -77,14 +82,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   float *sm = reinterpret_cast<float *>(smem4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // forward / reverse: points 2 pg, 2 pg + 1, 32 + 2 pg, 33 + 2 pg; columns 4 cg .. 4 cg + 3
-  const int pg = (lane & 7) + 8 * (warp & 1), cg = (lane >> 3) + 4 * (warp >> 1);
+  const int pg = ((lane >> 1) & 1) + ((lane >> 2) & 2) + 4 * (warp & 3);
+  const int cg = (lane & 1) + ((lane >> 1) & 2) + ((lane >> 2) & 4) + 8 * (warp >> 2);
   // weight gradients: rows pg + 16 i, columns cg + 16 j
   const int skip = prm.skip;
   const float beta = prm.beta, inv_beta = 1.0f / prm.beta;
   const bool weights = prm.g_partial != nullptr;
 
   for (int i = tid; i < (L - 1) * kW * kW; i += kThreads)
-    sm[M::w + (i / kW) * kWRow + i % kW] = prm.bwd[i];
+    sm[M::w + swizzled(i / kW, (i % kW) >> 2) + (i & 3)] = prm.bwd[i];
   for (int i = tid; i < kW * 3; i += kThreads) sm[M::w0 + (i / 3) * 4 + i % 3] = prm.w0[i];
   for (int i = tid; i < L * kW; i += kThreads) sm[M::bias + i] = prm.bias[i];
   for (int i = tid; i < kW; i += kThreads) sm[M::wout + i] = prm.wout[i];
@@ -149,13 +155,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       } else {
-        const float *wl = sm + M::w + (l - 1) * kW * kWRow + 4 * cg * kWRow;
+        const float *wl = sm + M::w + (l - 1) * kW * kW;
         const float *xl = sm + M::a + (l - 1) * kW * kARow + 4 * pg;
 #pragma unroll 2
         for (int k = 0; k < kW; k += 4) {
           float4 w[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const float4 *>(wl + j * kWRow + k);
+          for (int j = 0; j < 4; ++j)
+            w[j] = *reinterpret_cast<const float4 *>(wl + swizzled(4 * cg + j, k >> 2));
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const float4 xa = *reinterpret_cast<const float4 *>(xl + (k + q) * kARow);
@@ -310,14 +317,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       // (hb, hdb) of layer l - 1: W_l^T (zb, zdb)
-      const float *wl = sm + M::w + (l - 1) * kW * kWRow + 4 * cg;
+      const float *wl = sm + M::w + (l - 1) * kW * kW;
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[j][i] = make_float2(0.f, 0.f);
 #pragma unroll 4
       for (int c = 0; c < kW; ++c) {
-        const float4 w = *reinterpret_cast<const float4 *>(wl + c * kWRow);
+        const float4 w = *reinterpret_cast<const float4 *>(wl + swizzled(c, cg));
         const float4 za = *reinterpret_cast<const float4 *>(zb + c * kARow + 4 * pg);
         const float4 zc = *reinterpret_cast<const float4 *>(zb + c * kARow + 4 * pg + 64);
 #pragma unroll
