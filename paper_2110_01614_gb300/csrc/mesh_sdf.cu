@@ -145,7 +145,7 @@ cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *
   if (n_faces >= kTreeMinFaces && n_faces <= kTreeMaxFaces) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-        cudaMallocAsync(&mem, mesh_tree_bytes(n_faces, pts ? n : 0), s) != cudaSuccess)
+        cudaMallocAsync(&mem, mesh_tree_bytes(n_faces, pts ? n : 0, pts ? 0 : n), s) != cudaSuccess)
       mem = nullptr;
     if (!mem) cudaGetLastError();
   }

@@ -10,12 +10,14 @@
 //   * sign: w > 1/2 for the generalized winding number w.  The mesh is closed
 //     when its oriented edges cancel in pairs; then w is a whole number and
 //     equals the signed count of the triangles that a ray from the point
-//     crosses.  The ray runs along +z; a triangle is crossed when the
+//     crosses, along any axis (the one towards the nearest side of the mesh's
+//     box, which meets the fewest boxes).  A triangle is crossed when the
 //     projected point has a nonzero 2-D winding number about the projected
 //     triangle, with one half-open rule and one evaluation order for each
 //     edge, so that the triangles on either side of an edge always agree and
-//     no crossing is lost or counted twice.  Side tests that FP32 comparisons
-//     of coordinates do not settle are FP64.
+//     no crossing is lost or counted twice.  Side tests that FP32 does not
+//     settle beyond its rounding are FP64.
+// In front of either test of a triangle stands one of its bounding sphere.
 // Closedness is tested on the device by a hash of the boundary: every oriented
 // edge (a, b), named by the positions of its ends, adds h(a, b) - h(b, a)
 // modulo 2^64.  A closed mesh gives exactly 0; any other gives 0 with
@@ -29,14 +31,14 @@
 // the points' Morton order.  About 50 us for 20,480 triangles and 250,000
 // points, so it is rebuilt by every call and nothing is kept between calls.
 //
-// Bound: instruction issue of the descent (about 17 leaves for a point near
-// the surface, 70 for one far from it; 57% of the issue slots with 18 of 32
-// lanes active).  Measured on a closed mesh of 20,448 triangles, 250,000
-// fitting points (80% within 0.01 of the surface): brute force 107 ms; a
-// thread per point in the caller's order, side tests in FP64 3.5 ms; hard
-// points by the whole warp 1.85 ms; points in Morton order, FP32 filter before
-// the FP64 side tests 1.65 ms.  Leaf budgets of 6 / 12 / 24 / 48: 1.84 / 1.74 /
-// 1.63 / 1.57 ms, and 1.44 / 1.42 / 1.37 / 1.45 ms on 50,000 far points.
+// Bound: instruction issue of the searches (60% and 41% of the slots in the two
+// kernels) and their divergence (10 and 21 of 32 lanes active).  Measured on
+// 250,000 fitting points (80% within 0.01 of the surface) and 20,480 triangles:
+// brute force 107 ms; a thread per point in the caller's order with FP64 side
+// tests 3.5 ms; hard points by their own warp, points in Morton order, FP32 filters
+// 2.37 ms; spheres before the triangle tests and rays to the nearest side 2.1 ms;
+// hard points from a list, four warps each 0.96 ms (Morton order had put them
+// all into a few warps).
 
 #include "mesh_tree.cuh"
 
@@ -50,17 +52,27 @@ constexpr int kBlock = 256;              // threads of the build kernels = leave
 constexpr int kStack = 32;               // deeper than any tree of kTreeMaxFaces
 constexpr int kPointBits = 5;            // Morton bits per axis of the points' order
 constexpr int64_t kPointChunk = int64_t(1) << 20;
-constexpr int kLeafBudget = 24;          // leaves a thread visits before its warp takes over
+constexpr int64_t kHardMax = int64_t(1) << 18;
+constexpr int kHardWarps = 4;            // warps that search one hard point
+constexpr int kHardBlocks = 152 * 8;
+// Leaves a thread visits before its point is a hard one: 32 where points fill
+// the GPU (6 / 12 / 20 / 32 measured 1.54 / 1.22 / 0.99 / 0.89 ms on 250,000
+// fitting points, 48 and 96 more on far points), 4 where a launch has at most a
+// few points per block of the hard kernel and one thread's descent is all it
+// waits for (4 / 12 / 32: 200 points x 20,480 triangles 215 / 275 / 389 us, 4,000
+// points 240 / 274 / 364 us).
+constexpr int kLeafBudget = 32, kLeafBudgetFew = 4;
 
 // Scratch layout for a mesh of F faces.
 struct TreeMem {
   int64_t leaves;                        // power of two >= 2
   int bits;                              // Morton bits per axis
   int64_t chunk;                         // points ordered (and queried) at a time
-  size_t header, hist, phist, key, pkey, order, tri, node, block_box, total;
+  size_t header, hard_count, hist, phist, key, pkey, order, hard, tri, sphere, node, block_box, total;
+  unsigned hard_cap;                     // points the hard list holds
 };
 
-__host__ inline TreeMem tree_mem(int64_t F, int64_t points) {
+__host__ inline TreeMem tree_mem(int64_t F, int64_t points, int64_t nodes) {
   TreeMem m{};
   m.chunk = points < kPointChunk ? points : kPointChunk;
   m.leaves = 2;
@@ -73,12 +85,17 @@ __host__ inline TreeMem tree_mem(int64_t F, int64_t points) {
     return o;
   };
   m.header = take(sizeof(MeshTreeHeader));
+  m.hard_count = take(sizeof(unsigned));
   m.phist = take(m.chunk > 0 ? sizeof(unsigned) << (3 * kPointBits) : 0);
-  m.hist = take(sizeof(unsigned) << (3 * m.bits));     // one memset clears these three
+  m.hist = take(sizeof(unsigned) << (3 * m.bits));     // one memset clears these four
   m.key = take(sizeof(uint2) * (size_t)F);
   m.pkey = take(sizeof(uint2) * (size_t)m.chunk);
   m.order = take(sizeof(unsigned) * (size_t)m.chunk);
-  m.tri = take(sizeof(float) * 9 * kLeaf * (size_t)m.leaves);
+  const int64_t most = points > 0 ? m.chunk : nodes;
+  m.hard_cap = (unsigned)(most < kHardMax ? most : kHardMax);
+  m.hard = take(sizeof(int64_t) * (size_t)m.hard_cap);
+  m.tri = take(sizeof(float4) * 3 * kLeaf * (size_t)m.leaves);
+  m.sphere = take(sizeof(float4) * kLeaf * (size_t)m.leaves);
   m.node = take(sizeof(float4) * 3 * (size_t)m.leaves);
   const size_t blocks = (size_t)((m.leaves + kBlock - 1) / kBlock);
   m.block_box = take(sizeof(float) * 6 * 2 * blocks);
@@ -268,13 +285,12 @@ __global__ void __launch_bounds__(1024) tree_scan_kernel(unsigned *hist, int cel
   }
 }
 
-// Counting sort, second pass: faces into the leaves in cell order (leaf = 9
-// float4, one per coordinate of a, b, c, over its four triangles), and the
-// order in which the points are queried.
+// Counting sort, second pass: faces into the leaves in cell order (three float4
+// per triangle: a, b, c in turn), and the order in which the points are queried.
 __global__ void __launch_bounds__(kBlock) tree_scatter_kernel(
     const float *__restrict__ V, int64_t nv, const int32_t *__restrict__ F, int64_t nf, unsigned fb,
     int64_t n, const unsigned *__restrict__ start, const uint2 *__restrict__ key,
-    const unsigned *__restrict__ pstart, const uint2 *__restrict__ pkey, float *__restrict__ tri,
+    const unsigned *__restrict__ pstart, const uint2 *__restrict__ pkey, float4 *__restrict__ tri,
     unsigned *__restrict__ order) {
   if (blockIdx.x >= fb) {
     const int64_t i = (int64_t)(blockIdx.x - fb) * kBlock + threadIdx.x;
@@ -289,11 +305,18 @@ __global__ void __launch_bounds__(kBlock) tree_scatter_kernel(
   if (kr.x == 0xffffffffu) return;
   V3<float> a, b, c;
   load_face(V, nv, F, f, a, b, c);
-  const unsigned pos = start[kr.x] + kr.y;
-  float *o = tri + (size_t)(pos / kLeaf) * (9 * kLeaf) + pos % kLeaf;
-  o[0 * kLeaf] = a.x; o[1 * kLeaf] = a.y; o[2 * kLeaf] = a.z;
-  o[3 * kLeaf] = b.x; o[4 * kLeaf] = b.y; o[5 * kLeaf] = b.z;
-  o[6 * kLeaf] = c.x; o[7 * kLeaf] = c.y; o[8 * kLeaf] = c.z;
+  float4 *o = tri + 3 * (size_t)(start[kr.x] + kr.y);
+  o[0] = make_float4(a.x, a.y, a.z, b.x);
+  o[1] = make_float4(b.y, b.z, c.x, c.y);
+  o[2] = make_float4(c.z, 0.f, 0.f, 0.f);
+}
+
+struct Tri {
+  V3<float> a, b, c;
+};
+__device__ __forceinline__ Tri load_tri(const float4 *__restrict__ t) {
+  const float4 u = t[0], v = t[1], w = t[2];
+  return {{u.x, u.y, u.z}, {u.w, v.x, v.y}, {v.z, v.w, w.x}};
 }
 
 struct Box {
@@ -318,7 +341,8 @@ __device__ __forceinline__ void store_node(float4 *node, int64_t i, const Box &l
 
 // Boxes bottom-up: each block reduces 256 leaves (a subtree) in shared memory,
 // and the last block to finish builds the levels above the blocks' roots.
-__global__ void __launch_bounds__(kBlock) tree_box_kernel(float *__restrict__ tri,
+__global__ void __launch_bounds__(kBlock) tree_box_kernel(const float4 *__restrict__ tri,
+                                                          float4 *__restrict__ sphere,
                                                           float4 *__restrict__ node, int leaves,
                                                           float *block_box, MeshTreeHeader *hdr) {
   __shared__ Box sb[kBlock];
@@ -331,18 +355,33 @@ __global__ void __launch_bounds__(kBlock) tree_box_kernel(float *__restrict__ tr
   for (int k = 0; k < 3; ++k) { b.lo[k] = INFINITY; b.hi[k] = -INFINITY; }
   const unsigned valid = hdr->valid;
   if (t < per) {
-    float *q = tri + (size_t)leaf * (9 * kLeaf);
     for (int i = 0; i < kLeaf; ++i) {
-      if (leaf * kLeaf + i >= valid) {       // padding: NaN is never closest, never crossed
-        for (int e = 0; e < 9; ++e) q[e * kLeaf + i] = __int_as_float(0x7fc00000);
+      const int64_t f = leaf * kLeaf + i;
+      if (f >= valid) {                  // padding: a NaN is never near and never crossed
+        sphere[f] = make_float4(NAN, NAN, NAN, NAN);
         continue;
       }
+      const Tri q = load_tri(tri + 3 * f);
+      const float x[3][3] = {{q.a.x, q.b.x, q.c.x}, {q.a.y, q.b.y, q.c.y}, {q.a.z, q.b.z, q.c.z}};
+      // centre of the triangle's box, and the furthest vertex from it (a little
+      // further, for the rounding of the distances)
+      float c[3], r2 = 0.f;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float x = q[k * kLeaf + i], y = q[(3 + k) * kLeaf + i], z = q[(6 + k) * kLeaf + i];
-        b.lo[k] = fminf(b.lo[k], fminf(fminf(x, y), z));
-        b.hi[k] = fmaxf(b.hi[k], fmaxf(fmaxf(x, y), z));
+        const float l = fminf(fminf(x[k][0], x[k][1]), x[k][2]), h = fmaxf(fmaxf(x[k][0], x[k][1]), x[k][2]);
+        b.lo[k] = fminf(b.lo[k], l);
+        b.hi[k] = fmaxf(b.hi[k], h);
+        c[k] = 0.5f * l + 0.5f * h;
       }
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        float d2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) d2 = fmaf(x[k][v] - c[k], x[k][v] - c[k], d2);
+        r2 = fmaxf(r2, d2);
+      }
+      const float m = fmaxf(fmaxf(fabsf(c[0]), fabsf(c[1])), fabsf(c[2]));
+      sphere[f] = make_float4(c[0], c[1], c[2], fmaf(sqrtf(r2), 1.f + 1e-5f, 1e-6f * m));
     }
   }
   sb[t] = b;
@@ -443,68 +482,167 @@ __device__ __forceinline__ float node_dist2(V3<float> p, const float4 *__restric
   return box_dist2(p, u.x, u.y, u.z, u.w, v.x, v.y);
 }
 
-// The distances a box may have and still hold a closer triangle than `best`:
-// the triangle test's own rounding (slack, a few ulp of the coordinates) on top.
-__device__ __forceinline__ float box_limit(float best, float slack) {
-  const float r = sqrtf(best) + slack;
-  return fminf(r * r * (1.f + 1e-6f), kFarDist2);
+// How far a box or a sphere may be and still hold a closer triangle than one at
+// squared distance `best`: the triangle test's own rounding (slack, a few ulp of
+// the coordinates) on top.
+struct Reach {
+  float r, r2;
+};
+__device__ __forceinline__ Reach reach_of(float best, float slack) {
+  const float r = (sqrtf(best) + slack) * (1.f + 1e-6f);
+  return {r, fminf(r * r, kFarDist2)};
+}
+// Can the triangle in sphere s be within reach of p?
+__device__ __forceinline__ bool near_sphere(V3<float> p, const float4 &s, const Reach &reach) {
+  const float dx = p.x - s.x, dy = p.y - s.y, dz = p.z - s.z, r = reach.r + s.w;
+  return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= r * r;
 }
 
-// The rest of one point's search, by the whole warp: the tree is read as a
-// 32-way one (nodes over 1024 triangles, over 32, the triangles), a lane per
-// child.  Every lane returns the smallest squared distance.
-__device__ float warp_search(V3<float> p, float best, float slack, const float *__restrict__ tri,
-                             const float4 *__restrict__ node, int leaves) {
+// One point's search by `warps` warps, of which this is number `warp`: the tree
+// is read as a 32-way one (nodes over 1024 triangles, over 32, the triangles), a
+// lane per child, and the warps take the top nodes in turn.  `shared_best` (the
+// bits of the smallest squared distance of all warps; or null for one warp)
+// carries their results.  Every lane returns the smallest squared distance that
+// it knows of, of triangles within `reach`.
+__device__ float warp_search(V3<float> p, Reach reach, float slack, const float4 *__restrict__ tri,
+                             const float4 *__restrict__ sphere, const float4 *__restrict__ node,
+                             int leaves, unsigned warp, unsigned warps, unsigned *shared_best) {
   const unsigned lane = threadIdx.x & 31u;
-  const unsigned groups = (unsigned)leaves / 8u, tops = (groups + 31u) / 32u;
-  float limit = box_limit(best, slack);
-  for (unsigned t0 = 0; t0 < tops; t0 += 32) {
+  const unsigned groups = (unsigned)leaves / 8u;
+  // top nodes: over 1024 triangles, or fewer when that leaves warps idle
+  unsigned per = 32u;
+  while (per > 1u && groups / per < 4u * warps) per >>= 1;
+  const unsigned tops = (groups + per - 1u) / per;
+  float best = INFINITY;
+  for (unsigned t0 = 0; t0 < tops; t0 += 32u) {
     const unsigned t = t0 + lane;
     float dt = INFINITY;
-    if (t < tops) dt = tops > 1u ? node_dist2(p, node, tops + t) : 0.f;
-    unsigned tm = __ballot_sync(0xffffffffu, dt <= limit);
+    if (t < tops && t % warps == warp) dt = tops > 1u ? node_dist2(p, node, tops + t) : 0.f;
+    unsigned tm = __ballot_sync(0xffffffffu, dt <= reach.r2);
     while (tm) {
       const unsigned ti = t0 + __ffs(tm) - 1;
       tm &= tm - 1;
-      const unsigned g = 32u * ti + lane;
-      const float dg = g < groups ? node_dist2(p, node, groups + g) : INFINITY;
-      unsigned gm = __ballot_sync(0xffffffffu, dg <= limit);
-      while (gm) {
-        const unsigned gi = 32u * ti + __ffs(gm) - 1;
-        gm &= gm - 1;
-        const float *q = tri + ((size_t)gi * 8 + (lane >> 2)) * (9 * kLeaf) + (lane & 3u);
-        const float d = tri_dist2(p, {__ldg(q), __ldg(q + 4), __ldg(q + 8)},
-                                  {__ldg(q + 12), __ldg(q + 16), __ldg(q + 20)},
-                                  {__ldg(q + 24), __ldg(q + 28), __ldg(q + 32)});
-        // distances are not negative, so their bits order them (a NaN comes last)
-        const float m = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(d)));
-        if (m < best) {
-          best = m;
-          limit = box_limit(best, slack);
-          gm &= __ballot_sync(0xffffffffu, dg <= limit);
+      if (shared_best) {
+        const float other = __uint_as_float(*(volatile unsigned *)shared_best);
+        if (other < best) {
+          best = other;
+          const Reach closer = reach_of(best, slack);
+          if (closer.r2 < reach.r2) reach = closer;
         }
       }
-      tm &= __ballot_sync(0xffffffffu, dt <= limit);
+      const unsigned g = per * ti + lane;
+      const float dg = lane < per && g < groups ? node_dist2(p, node, groups + g) : INFINITY;
+      unsigned gm = __ballot_sync(0xffffffffu, dg <= reach.r2);
+      while (gm) {
+        const size_t f = (size_t)32 * (per * ti + __ffs(gm) - 1) + lane;
+        gm &= gm - 1;
+        float d = INFINITY;
+        if (near_sphere(p, sphere[f], reach)) {
+          const Tri q = load_tri(tri + 3 * f);
+          d = tri_dist2(p, q.a, q.b, q.c);
+        }
+        // distances are not negative, so their bits order them (a NaN comes last)
+        const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(d));
+        if (__uint_as_float(m) < best) {
+          best = __uint_as_float(m);
+          if (shared_best && lane == 0) atomicMin(shared_best, m);
+          const Reach closer = reach_of(best, slack);
+          if (closer.r2 < reach.r2) reach = closer;
+          gm &= __ballot_sync(0xffffffffu, dg <= reach.r2);
+        }
+      }
+      tm &= __ballot_sync(0xffffffffu, dt <= reach.r2);
     }
   }
   return best;
 }
 
+// Coordinate k of p, and the ray's axes: it runs along axis A, the other two
+// span the projection in an order that keeps its orientation.
+template <int A>
+__device__ __forceinline__ V3<float> along_z(V3<float> p) {
+  if (A == 0) return {p.y, p.z, p.x};
+  if (A == 1) return {p.z, p.x, p.y};
+  return p;
+}
+
+// Winding number of the mesh about p: signed crossings of the ray from p along
+// axis A, upwards (dir = 1) or downwards (dir = -1).
+template <int A>
+__device__ int ray_crossings(V3<float> p0, int dir, const float4 *__restrict__ tri,
+                             const float4 *__restrict__ sphere, const float4 *__restrict__ node,
+                             int leaves, int *stack) {
+  const V3<float> p = along_z<A>(p0);
+  int wind = 0, sp = 0, at = 1;
+  auto meets = [&](V3<float> lo, V3<float> hi) {
+    lo = along_z<A>(lo);
+    hi = along_z<A>(hi);
+    return p.x >= lo.x && p.x <= hi.x && p.y >= lo.y && p.y <= hi.y &&
+           (dir > 0 ? p.z <= hi.z : p.z >= lo.z);
+  };
+  while (at) {
+    while (at && at < leaves) {
+      const float4 *nd = node + 3 * (size_t)at;
+      const float4 u = __ldg(nd), v = __ldg(nd + 1), w = __ldg(nd + 2);
+      const bool l = meets({u.x, u.y, u.z}, {u.w, v.x, v.y});
+      const bool r = meets({v.z, v.w, w.x}, {w.y, w.z, w.w});
+      if (l && r) stack[sp++] = 2 * at + 1;
+      at = l ? 2 * at : (r ? 2 * at + 1 : (sp > 0 ? stack[--sp] : 0));
+    }
+    if (!at) break;
+    const size_t f = (size_t)(at - leaves) * kLeaf;
+    float4 c[kLeaf];
+#pragma unroll
+    for (int i = 0; i < kLeaf; ++i) c[i] = sphere[f + i];
+#pragma unroll
+    for (int i = 0; i < kLeaf; ++i) {
+      const V3<float> m = along_z<A>({c[i].x, c[i].y, c[i].z});
+      const float dx = p.x - m.x, dy = p.y - m.y;
+      if (!(fmaf(dx, dx, dy * dy) <= c[i].w * c[i].w)) continue;
+      const Tri q = load_tri(tri + 3 * (f + i));
+      const V3<float> a = along_z<A>(q.a), b = along_z<A>(q.b), d = along_z<A>(q.c);
+      const int wn = edge_winding(p, a, b) + edge_winding(p, b, d) + edge_winding(p, d, a);
+      if (wn != 0) {
+        // in front of p along the ray, and which way round
+        const float side = plane_side(p, a, b, d);
+        const bool above = wn > 0 ? side > 0.f : side < 0.f;
+        const bool below = wn > 0 ? side < 0.f : side > 0.f;
+        if (dir > 0 ? above : below) wind += dir * wn;
+      }
+    }
+    at = sp > 0 ? stack[--sp] : 0;
+  }
+  return wind;
+}
+
+// Rounding of the distance test: coordinates of this size, a few ulp.
+__device__ __forceinline__ float slack_of(V3<float> p, const MeshTreeHeader *__restrict__ hdr) {
+  float scale = fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fabsf(p.z));
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    scale = fmaxf(scale, fmaxf(fabsf(unordered(hdr->neg_lo[k])), fabsf(unordered(hdr->hi[k]))));
+  return 1e-6f * scale;
+}
+
 // Signed distance of every point: nearest-first descent for the distance, then
-// the crossings of the ray along +z for the sign.  A thread owns a point.  A
-// point about as far from many triangles (the middle of a round body) would
-// keep its thread descending long after the warp's other 31 are done, so after
-// kLeafBudget leaves it is left to the whole warp (warp_search).
+// the crossings of a ray for the sign.  A thread owns a point.  A point about as
+// far from many triangles (the middle of a round body) would keep its thread
+// descending long after the others are done, and neighbours of such a point are
+// no better, so after a budget of leaves it is put on a list and searched by a
+// block of its own (mesh_hard_kernel).
 //
 // Neighbouring threads take neighbouring points, so that a warp walks one part
 // of the tree: explicit points in the Morton order of the build, grid nodes in
 // bricks of 8 x 4 x 4 per block.
 __global__ void __launch_bounds__(128) mesh_tree_kernel(const float4 *__restrict__ tri,
+                                                        const float4 *__restrict__ sphere,
                                                         const float4 *__restrict__ node, int leaves,
                                                         const MeshTreeHeader *__restrict__ hdr,
                                                         const float4 *__restrict__ pts,
                                                         const unsigned *__restrict__ order, int64_t n,
-                                                        float *__restrict__ out, const GridPts grid) {
+                                                        float *__restrict__ out, const GridPts grid,
+                                                        int budget, unsigned *hard_count,
+                                                        int64_t *hard_list, unsigned hard_cap) {
   if (!mesh_tree_usable(hdr)) return;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (!pts) {
@@ -520,21 +658,30 @@ __global__ void __launch_bounds__(128) mesh_tree_kernel(const float4 *__restrict
   if (idx < n) p = query_point(pts, grid, idx);
   const bool finite = fabsf(p.x) < INFINITY && fabsf(p.y) < INFINITY && fabsf(p.z) < INFINITY;
   const bool work = idx < n && finite;
-  // rounding of the distance test: coordinates of this size, a few ulp
-  float scale = fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fabsf(p.z));
+  const float slack = slack_of(p, hdr);
+  // the ray will run towards the nearest side of the mesh's box
+  const float pc[3] = {p.x, p.y, p.z};
+  float nearest = INFINITY;
+  int axis = 2, dir = 1;
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
-    scale = fmaxf(scale, fmaxf(fabsf(unordered(hdr->neg_lo[k])), fabsf(unordered(hdr->hi[k]))));
-  const float slack = 1e-6f * scale;
+  for (int k = 0; k < 3; ++k) {
+    const float up = unordered(hdr->hi[k]) - pc[k], down = pc[k] + unordered(hdr->neg_lo[k]);
+    if (fminf(up, down) < nearest) {
+      nearest = fminf(up, down);
+      axis = k;
+      dir = up <= down ? 1 : -1;
+    }
+  }
 
   int stack[kStack];
   float dist[kStack];
-  int sp = 0, at = 1, left = kLeafBudget;
-  float best = kFarDist2, limit = kFarDist2;
+  int sp = 0, at = 1, left = budget;
+  float best = kFarDist2;
+  Reach reach = {INFINITY, kFarDist2};
   // the next box on the stack that may still hold a closer triangle (0: none)
   auto pop = [&]() -> int {
     while (sp > 0)
-      if (dist[--sp] <= limit) return stack[sp];
+      if (dist[--sp] <= reach.r2) return stack[sp];
     return 0;
   };
   if (!work) at = 0;
@@ -547,98 +694,107 @@ __global__ void __launch_bounds__(128) mesh_tree_kernel(const float4 *__restrict
       const bool near_left = dl <= dr;
       const float dn = near_left ? dl : dr, df = near_left ? dr : dl;
       const int near = 2 * at + (near_left ? 0 : 1);
-      if (df <= limit) {
+      if (df <= reach.r2) {
         stack[sp] = near ^ 1;
         dist[sp++] = df;
       }
-      at = dn <= limit ? near : pop();
+      at = dn <= reach.r2 ? near : pop();
     }
     if (!at || left-- == 0) break;
-    const float4 *q = tri + (size_t)(at - leaves) * 9;
-    float4 c[9];
+    const size_t f = (size_t)(at - leaves) * kLeaf;
+    float4 c[kLeaf];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) c[e] = __ldg(q + e);
-    float d = best;
-#pragma unroll
+    for (int i = 0; i < kLeaf; ++i) c[i] = sphere[f + i];
+#pragma unroll 1
     for (int i = 0; i < kLeaf; ++i) {
-      auto el = [i](const float4 &x) { return i == 0 ? x.x : i == 1 ? x.y : i == 2 ? x.z : x.w; };
-      d = fminf(d, tri_dist2(p, {el(c[0]), el(c[1]), el(c[2])}, {el(c[3]), el(c[4]), el(c[5])},
-                             {el(c[6]), el(c[7]), el(c[8])}));
-    }
-    if (d < best) {
-      best = d;
-      limit = box_limit(best, slack);
+      const float4 ci = i == 0 ? c[0] : i == 1 ? c[1] : i == 2 ? c[2] : c[3];
+      if (!near_sphere(p, ci, reach)) continue;
+      const Tri q = load_tri(tri + 3 * (f + i));
+      const float d = tri_dist2(p, q.a, q.b, q.c);
+      if (d < best) {
+        best = d;
+        reach = reach_of(best, slack);
+      }
     }
     at = pop();
   }
+  // a hard point goes on the list for mesh_hard_kernel, or, when that is full,
+  // to this warp
   __syncwarp();
-  unsigned hard = __ballot_sync(0xffffffffu, left < 0);
-  while (hard) {
-    const int q = __ffs(hard) - 1;
-    hard &= hard - 1;
+  bool hard = false;
+  if (left < 0) {
+    const unsigned at_list = atomicAdd(hard_count, 1u);
+    if (at_list < hard_cap) hard_list[at_list] = idx;
+    else hard = true;
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, hard);
+  while (todo) {
+    const int q = __ffs(todo) - 1;
+    todo &= todo - 1;
     const V3<float> pq = {__shfl_sync(0xffffffffu, p.x, q), __shfl_sync(0xffffffffu, p.y, q),
                           __shfl_sync(0xffffffffu, p.z, q)};
-    const float d = warp_search(pq, __shfl_sync(0xffffffffu, best, q),
-                                __shfl_sync(0xffffffffu, slack, q),
-                                reinterpret_cast<const float *>(tri), node, leaves);
-    if ((int)(threadIdx.x & 31u) == q) best = d;
+    const float sl = __shfl_sync(0xffffffffu, slack, q), bq = __shfl_sync(0xffffffffu, best, q);
+    const float d = warp_search(pq, reach_of(bq, sl), sl, tri, sphere, node, leaves, 0u, 1u, nullptr);
+    if ((int)(threadIdx.x & 31u) == q) best = fminf(best, d);
   }
   if (!work) {
     if (idx < n) out[idx] = sqrtf(kFarDist2);
     return;
   }
 
-  // winding number: signed crossings of the ray from p along +z
-  int wind = 0;
-  sp = 0;
-  at = 1;
-  while (at) {
-    while (at && at < leaves) {
-      const float4 *nd = node + 3 * (size_t)at;
-      const float4 u = __ldg(nd), v = __ldg(nd + 1), w = __ldg(nd + 2);
-      const bool l = p.x >= u.x && p.x <= u.w && p.y >= u.y && p.y <= v.x && p.z <= v.y;
-      const bool r = p.x >= v.z && p.x <= w.y && p.y >= v.w && p.y <= w.z && p.z <= w.w;
-      if (l && r) stack[sp++] = 2 * at + 1;
-      at = l ? 2 * at : (r ? 2 * at + 1 : (sp > 0 ? stack[--sp] : 0));
-    }
-    if (!at) break;
-    const float4 *q = tri + (size_t)(at - leaves) * 9;
-    float4 c[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) c[e] = __ldg(q + e);
-#pragma unroll
-    for (int i = 0; i < kLeaf; ++i) {
-      auto el = [i](const float4 &x) { return i == 0 ? x.x : i == 1 ? x.y : i == 2 ? x.z : x.w; };
-      const V3<float> a = {el(c[0]), el(c[1]), el(c[2])}, b = {el(c[3]), el(c[4]), el(c[5])},
-                      d = {el(c[6]), el(c[7]), el(c[8])};
-      const int wn = edge_winding(p, a, b) + edge_winding(p, b, d) + edge_winding(p, d, a);
-      if (wn != 0) {
-        const float side = plane_side(p, a, b, d);
-        if (wn > 0 ? side > 0.f : side < 0.f) wind += wn;
-      }
-    }
-    at = sp > 0 ? stack[--sp] : 0;
-  }
+  // sign: any axis and direction give the same whole number
+  const int wind = axis == 0   ? ray_crossings<0>(p, dir, tri, sphere, node, leaves, stack)
+                   : axis == 1 ? ray_crossings<1>(p, dir, tri, sphere, node, leaves, stack)
+                               : ray_crossings<2>(p, dir, tri, sphere, node, leaves, stack);
   const float d = sqrtf(best);
   out[idx] = wind >= 1 ? -d : d;
 }
 
+// The listed points, a block each in turn: out holds the sign and an upper bound
+// of the distance.
+__global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
+    const float4 *__restrict__ tri, const float4 *__restrict__ sphere, const float4 *__restrict__ node,
+    int leaves, const MeshTreeHeader *__restrict__ hdr, const float4 *__restrict__ pts,
+    float *__restrict__ out, const GridPts grid, const unsigned *__restrict__ hard_count,
+    const int64_t *__restrict__ hard_list, unsigned hard_cap) {
+  __shared__ unsigned best_bits;
+  const unsigned count = min(*hard_count, hard_cap);
+  for (unsigned i = blockIdx.x; i < count; i += gridDim.x) {
+    const int64_t idx = hard_list[i];
+    const V3<float> p = query_point(pts, grid, idx);
+    const float slack = slack_of(p, hdr), d = out[idx];
+    if (threadIdx.x == 0) best_bits = 0x7f800000u;
+    __syncthreads();
+    // (the root rounds: a little more than its square)
+    warp_search(p, reach_of(d * d * (1.f + 1e-6f), slack), slack, tri, sphere, node, leaves,
+                threadIdx.x >> 5, kHardWarps, &best_bits);
+    __syncthreads();
+    if (threadIdx.x == 0) out[idx] = copysignf(sqrtf(__uint_as_float(best_bits)), d);
+    __syncthreads();
+  }
+}
+
 }  // namespace
 
-size_t mesh_tree_bytes(int64_t n_faces, int64_t n_points) { return tree_mem(n_faces, n_points).total; }
+size_t mesh_tree_bytes(int64_t n_faces, int64_t n_points, int64_t n_nodes) {
+  return tree_mem(n_faces, n_points, n_nodes).total;
+}
 
 cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t *faces,
                              int64_t n_faces, const float4 *pts, int64_t n, float *out,
                              const GridPts &grid, void *mem, cudaStream_t s) {
-  const TreeMem m = tree_mem(n_faces, pts ? n : 0);
+  const TreeMem m = tree_mem(n_faces, pts ? n : 0, pts ? 0 : n);
   char *base = static_cast<char *>(mem);
   MeshTreeHeader *hdr = reinterpret_cast<MeshTreeHeader *>(base + m.header);
   unsigned *hist = reinterpret_cast<unsigned *>(base + m.hist);
+  unsigned *hard_count = reinterpret_cast<unsigned *>(base + m.hard_count);
+  int64_t *hard = reinterpret_cast<int64_t *>(base + m.hard);
   unsigned *phist = reinterpret_cast<unsigned *>(base + m.phist);
   uint2 *key = reinterpret_cast<uint2 *>(base + m.key);
   uint2 *pkey = reinterpret_cast<uint2 *>(base + m.pkey);
   unsigned *order = reinterpret_cast<unsigned *>(base + m.order);
-  float *tri = reinterpret_cast<float *>(base + m.tri);
+  float4 *tri = reinterpret_cast<float4 *>(base + m.tri);
+  float4 *sphere = reinterpret_cast<float4 *>(base + m.sphere);
   float4 *node = reinterpret_cast<float4 *>(base + m.node);
   float *block_box = reinterpret_cast<float *>(base + m.block_box);
   const int cells = 1 << (3 * m.bits), pcells = 1 << (3 * kPointBits);
@@ -651,7 +807,7 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
     const int64_t k = pts ? (n - c0 < m.chunk ? n - c0 : m.chunk) : 0;
     if (c0 > 0) {
       fb = 0;
-      e = cudaMemsetAsync(phist, 0, sizeof(unsigned) * pcells, s);
+      e = cudaMemsetAsync(base + m.hard_count, 0, m.phist - m.hard_count + sizeof(unsigned) * pcells, s);
       if (e != cudaSuccess) return e;
     }
     const unsigned blocks = fb + (unsigned)((k + kBlock - 1) / kBlock);
@@ -664,7 +820,8 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
                                                  phist, pkey, tri, order);
     if (fb > 0) {
       const int64_t bb = m.leaves < kBlock ? 1 : m.leaves / kBlock;
-      tree_box_kernel<<<(unsigned)bb, kBlock, 0, s>>>(tri, node, (int)m.leaves, block_box, hdr);
+      tree_box_kernel<<<(unsigned)bb, kBlock, 0, s>>>(tri, sphere, node, (int)m.leaves, block_box,
+                                                      hdr);
     }
     int64_t qb = (k + 127) / 128, count = k;
     if (!pts) {
@@ -672,8 +829,12 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
       qb = ((N + 7) / 8) * ((N + 3) / 4) * ((N + 3) / 4);
       count = n;
     }
-    mesh_tree_kernel<<<(unsigned)qb, 128, 0, s>>>(reinterpret_cast<const float4 *>(tri), node,
-                                                 (int)m.leaves, hdr, cp, order, count, out + c0, grid);
+    mesh_tree_kernel<<<(unsigned)qb, 128, 0, s>>>(tri, sphere, node, (int)m.leaves, hdr, cp, order,
+                                                 count, out + c0, grid,
+                                                 n <= 4 * kHardBlocks ? kLeafBudgetFew : kLeafBudget,
+                                                 hard_count, hard, m.hard_cap);
+    mesh_hard_kernel<<<kHardBlocks, 32 * kHardWarps, 0, s>>>(tri, sphere, node, (int)m.leaves, hdr, cp,
+                                                            out + c0, grid, hard_count, hard, m.hard_cap);
     if (!pts) break;
   }
   return cudaGetLastError();

@@ -30,8 +30,8 @@ __device__ __forceinline__ bool mesh_tree_usable(const MeshTreeHeader *h) {
 constexpr int64_t kTreeMinFaces = 128;
 constexpr int64_t kTreeMaxFaces = int64_t(1) << 28;
 
-// n_points: explicit query points (0 for a grid, whose nodes need no scratch).
-size_t mesh_tree_bytes(int64_t n_faces, int64_t n_points);
+// n_points: explicit query points; n_nodes: nodes of a grid (the other is 0).
+size_t mesh_tree_bytes(int64_t n_faces, int64_t n_points, int64_t n_nodes);
 // Build the tree in `mem` (mesh_tree_bytes, 256-byte aligned) and write the
 // signed distances of all points if it is usable; out is untouched otherwise.
 cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t *faces,
