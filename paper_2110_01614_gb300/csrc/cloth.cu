@@ -13,11 +13,12 @@
 // 1024: 7.4 us at 6.8 TB/s).  With an IEEE square root and division per spring
 // (about 60 instructions of 590 per vertex) the issue slots were 77% busy; the
 // reciprocal square root with one Newton step needs 14 and carries the same
-// FP32 rounding.  1024 x 1024: 20.5 -> 16.4 us with x and x_prev from DRAM, 12.4 us from L2; tiles of 32 x 8 vertices read
+// FP32 rounding.  1024 x 1024, x and x_prev from DRAM: 20.5 -> 16.4 us, 14.1 launched overlapped; tiles of 32 x 8 vertices read
 // 1.3 rows per row written.  Evaluating each spring once, in strips that pass
-// the scalars on by shuffles, measured 15.5 us (and 22.5 with the IEEE forms):
+// the scalars on by shuffles, measured 15.5 us against 12.4 with everything in L2:
 // the shuffles and the lower occupancy cost more than the springs.
 
+#include "launch.cuh"
 #include "nsdf_internal.h"
 
 namespace nsdf {
@@ -33,12 +34,14 @@ __device__ __forceinline__ float spring(float dx, float dy, float dz, float rest
   return d2 > 0.f ? k * fmaf(-rest, r, 1.0f) : 0.f;
 }
 
-__global__ void __launch_bounds__(kTileX *kTileY) cloth_step_kernel(const float4 *__restrict__ x,
-                                                                    float4 *__restrict__ xprev,
+// (Plain pointers: an invariant load might move ahead of the wait.)
+__global__ void __launch_bounds__(kTileX *kTileY) cloth_step_kernel(const float4 *x, float4 *xprev,
                                                                     int nx, int ny, float hx, float hz,
                                                                     float k, float g, float dt) {
   const int j = blockIdx.x * kTileX + threadIdx.x % kTileX;   // column (along x)
   const int i = blockIdx.y * kTileY + threadIdx.x / kTileX;   // row (along z)
+  wait_for_predecessor();
+  release_successor();
   if (j >= nx || i >= ny) return;
   const int64_t v = (int64_t)i * nx + j;
   const float4 p = x[v], pp = xprev[v];
@@ -81,8 +84,10 @@ extern "C" nsdf_status nsdf_cloth_step(const float *x, float *x_prev_inout, int 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const dim3 grid((unsigned)((nx + nsdf::kTileX - 1) / nsdf::kTileX),
                   (unsigned)((ny + nsdf::kTileY - 1) / nsdf::kTileY));
-  nsdf::cloth_step_kernel<<<grid, nsdf::kTileX * nsdf::kTileY, 0, s>>>(
-      reinterpret_cast<const float4 *>(x), reinterpret_cast<float4 *>(x_prev_inout), nx, ny, hx, hz,
-      k_over_m, g, dt);
-  return cudaGetLastError() == cudaSuccess ? NSDF_OK : NSDF_ERR_CUDA;
+  return nsdf::launch_overlapped(nsdf::cloth_step_kernel, grid, nsdf::kTileX * nsdf::kTileY, 0, s,
+                                 reinterpret_cast<const float4 *>(x),
+                                 reinterpret_cast<float4 *>(x_prev_inout), nx, ny, hx, hz, k_over_m,
+                                 g, dt) == cudaSuccess
+             ? NSDF_OK
+             : NSDF_ERR_CUDA;
 }

@@ -42,13 +42,14 @@
 // in f32x2 pairs and the weights arriving while L0 is computed.  Sums over the
 // 64 columns stay one chain in column order, which the second warpgroup takes
 // over from the first, so both kernels give the same bits.  4,096 points of
-// 3-64x3-1: 17.2 -> 12.3 us a call.  On large calls (1,048,576 points, grouped
+// 3-64x3-1: 17.2 -> 9.6 us a call (12.3 without the overlapped launch).  On large calls (1,048,576 points, grouped
 // scenes) that form measured 0.90-1.02 of this one's speed, with one or two
 // warpgroups per tile: the epilogues' latency, not their FP32 instructions,
 // bounds them.
 
 #include <cudaTypedefs.h>
 
+#include "launch.cuh"
 #include "nsdf_internal.h"
 #include "softplus.cuh"
 #include "tc_ptx.cuh"
@@ -550,6 +551,20 @@ __global__ void __launch_bounds__(256, 1)
   const long long budget = prm.wait_budget;
   volatile int no_abort = 0;
 
+  // set up beside the end of the kernel before this one
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  const uint32_t ncols = (uint32_t)cta_cols(L, 1);
+  if (tid < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     sbase + off_bar + 8),
+                 "r"(ncols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  wait_for_predecessor();
+  release_successor();
   // everything the tile needs is asked for at once
   const int64_t idx = (int64_t)blockIdx.x * kM + r;
   const bool valid = idx < prm.n;
@@ -564,21 +579,10 @@ __global__ void __launch_bounds__(256, 1)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + lay.wlo), "l"(prm.fwd16_lo + src));
   }
   asm volatile("cp.async.commit_group;\n");
-  for (int e = tid; e < kW * 3; e += 256) sW0[(e % 3) * kW + e / 3] = __ldg(prm.w0 + e);
-  for (int e = tid; e < L * kW; e += 256) sB[e] = __ldg(prm.bias + e);
-  for (int e = tid; e < kW; e += 256) sWo[e] = __ldg(prm.wout + e);
-  if (tid == 0) {
-    sBo[0] = __ldg(prm.bout);
-    mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  const uint32_t ncols = (uint32_t)cta_cols(L, 1);
-  if (tid < 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     sbase + off_bar + 8),
-                 "r"(ncols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-  }
+  for (int e = tid; e < kW * 3; e += 256) sW0[(e % 3) * kW + e / 3] = prm.w0[e];
+  for (int e = tid; e < L * kW; e += 256) sB[e] = prm.bias[e];
+  for (int e = tid; e < kW; e += 256) sWo[e] = prm.wout[e];
+  if (tid == 0) sBo[0] = prm.bout[0];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -739,8 +743,7 @@ cudaError_t launch_small_t(const QueryParams &p, int64_t tiles, cudaStream_t s) 
   cudaError_t e = cudaFuncSetAttribute(query_w64_small_kernel<kF16>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  query_w64_small_kernel<kF16><<<(int)tiles, 256, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(query_w64_small_kernel<kF16>, dim3((unsigned)tiles), 256, smem, s, p);
 }
 
 // Dynamic shared memory of a launch: the layout, plus padding so that no
