@@ -797,13 +797,10 @@ nsdf_status grouped_launch_tc16_ff(nsdf_ctx *ctx, const GroupedArgs &g, cudaStre
   const int grid = query_tc16_ff_grouped_grid(max_tiles, ctx->num_sms);
   nsdf_status st = ensure_scratch(ctx, query_tc16_ff_scratch_bytes(grid));
   if (st != NSDF_OK) return st;
-  cudaError_t e = launch_build_tile_list(g.offsets, g.counts, ctx->n_nets, 128, g.max_total,
-                                         ctx->d_tile_start, ctx->d_err, s, 2);
+  cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, 128,
+                                       g.max_total, ctx->d_tile_start, 2, g.T, ctx->d_body,
+                                       ctx->d_err, s);
   if (e != cudaSuccess) return map_err(e);
-  if (g.T) {
-    e = launch_body_transforms(g.T, ctx->n_nets, ctx->d_body, ctx->d_err, s);
-    if (e != cudaSuccess) return map_err(e);
-  }
   QueryParams p{};
   fill_net(ctx, 0, p);
   p.pts = reinterpret_cast<const float4 *>(g.pts);
@@ -826,13 +823,10 @@ nsdf_status grouped_launch_tc16_ff(nsdf_ctx *ctx, const GroupedArgs &g, cudaStre
 // network's tile count rounded up to even (the two warpgroups of a CTA take
 // a pair of tiles of one network); cps = CTAs per SM (0: as many as fit).
 nsdf_status grouped_launch_w64(nsdf_ctx *ctx, const GroupedArgs &g, int cps, cudaStream_t s) {
-  cudaError_t e = launch_build_tile_list(g.offsets, g.counts, ctx->n_nets, 128, g.max_total,
-                                         ctx->d_tile_start, ctx->d_err, s, 2);
+  cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, 128,
+                                       g.max_total, ctx->d_tile_start, 2, g.T, ctx->d_body,
+                                       ctx->d_err, s);
   if (e != cudaSuccess) return map_err(e);
-  if (g.T) {
-    e = launch_body_transforms(g.T, ctx->n_nets, ctx->d_body, ctx->d_err, s);
-    if (e != cudaSuccess) return map_err(e);
-  }
   QueryParams p{};
   fill_net(ctx, 0, p);
   p.pts = reinterpret_cast<const float4 *>(g.pts);
@@ -857,14 +851,10 @@ nsdf_status grouped_launch(nsdf_ctx *ctx, const GroupedArgs &g, int pt, int cps,
   const int grid = grouped_grid(ctx, pt, cps, g.max_total);
   nsdf_status st = ensure_scratch(ctx, fp32_scratch_bytes_pt(a.width, pt, a.n_hidden, grid));
   if (st != NSDF_OK) return st;
-  cudaError_t e = launch_build_tile_list(g.offsets, g.counts, ctx->n_nets,
-                                         fp32_tile_points(a.width, pt), g.max_total,
-                                         ctx->d_tile_start, ctx->d_err, s);
+  cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, fp32_tile_points(a.width, pt),
+                                       g.max_total, ctx->d_tile_start, 1, g.T, ctx->d_body,
+                                       ctx->d_err, s);
   if (e != cudaSuccess) return map_err(e);
-  if (g.T) {
-    e = launch_body_transforms(g.T, ctx->n_nets, ctx->d_body, ctx->d_err, s);
-    if (e != cudaSuccess) return map_err(e);
-  }
   QueryParams p{};
   fill_net(ctx, 0, p);
   p.pts = reinterpret_cast<const float4 *>(g.pts);

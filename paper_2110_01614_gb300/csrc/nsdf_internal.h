@@ -207,12 +207,12 @@ int64_t ctx_blob_offsets(const nsdf_ctx *ctx, int64_t *woff, int64_t *boff, int 
 void **ctx_train_slot(nsdf_ctx *ctx);
 void train_state_free(void *state);
 
-cudaError_t launch_build_tile_list(const int64_t *offsets, const int64_t *counts, int n_nets, int P,
-                                   int64_t max_total, int32_t *tile_start, int *err,
-                                   cudaStream_t s, int round_to = 1);
-// T [n_nets][16] (row-major 4x4 poses, device) -> out [n_nets][kBodyFloats]
-cudaError_t launch_body_transforms(const float *T, int n_nets, float *out, int *err,
-                                   cudaStream_t s);
+// Work list of a grouped launch (tile_start [n_nets + 1]) and, where T is not
+// null, the bodies' transforms: T [n_nets][16] (row-major 4x4 poses, device) ->
+// body [n_nets][kBodyFloats]
+cudaError_t launch_grouped_setup(const int64_t *offsets, const int64_t *counts, int n_nets, int P,
+                                 int64_t max_total, int32_t *tile_start, int round_to, const float *T,
+                                 float *body, int *err, cudaStream_t s);
 
 size_t backward_smem_bytes(int width, int n_hidden, int64_t n_params);
 bool backward_supported(int width, int n_hidden, int64_t n_params);

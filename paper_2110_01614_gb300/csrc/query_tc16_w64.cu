@@ -277,6 +277,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   // this thread's TMEM row: accumulator at column 0, slopes of layer j at 64 + 32 j
   const uint32_t tb = tmem + (uint32_t)(wg * tile_cols(L)) + ((uint32_t)(32 * q) << 16);
 
+  wait_for_predecessor();      // (a grouped launch: its work list)
+  release_successor();
   const bool grouped = prm.g_nets > 0;
   const int64_t tiles = grouped ? (int64_t)prm.g_tile_start[prm.g_nets] : (prm.n + kM - 1) / kM;
   const int64_t pairs = (tiles + 1) / 2;
@@ -337,19 +339,22 @@ __global__ void __launch_bounds__(kThreads, 2)
       const float *gbo = grouped ? prm.g_netptrs[k].bout : prm.bout;
       // 16-bit weights: row n of layer i (64 values = 8 chunks of 16 B) into
       // the 128-byte swizzle (chunk j of row n at j ^ (n % 8))
+#pragma unroll 2
       for (int e = tid; e < nh * kW * 8; e += kThreads) {
         const int i = e / (kW * 8), n = (e / 8) % kW, j = e % 8;
         const size_t src = ((size_t)i * kW + n) * kW + 8 * j;
         const int dst = i * kWBytes + n * 128 + ((j ^ (n & 7)) * 16);
-        *reinterpret_cast<uint4 *>(smem + lay.whi + dst) = __ldg(reinterpret_cast<const uint4 *>(w16 + src));
+        // (plain loads: an invariant one might move ahead of the wait above)
+        *reinterpret_cast<uint4 *>(smem + lay.whi + dst) = *reinterpret_cast<const uint4 *>(w16 + src);
         if constexpr (kSplit)
           *reinterpret_cast<uint4 *>(smem + lay.wlo + dst) =
-              __ldg(reinterpret_cast<const uint4 *>(w16lo + src));
+              *reinterpret_cast<const uint4 *>(w16lo + src);
       }
-      for (int e = tid; e < kW * 3; e += kThreads) sW0[e] = __ldg(gw0 + e);
-      for (int e = tid; e < L * kW; e += kThreads) sB[e] = __ldg(gb + e);
-      for (int e = tid; e < kW; e += kThreads) sWo[e] = __ldg(gwo + e);
-      if (tid == 0) sBo[0] = __ldg(gbo);
+      if (tid < kW * 3) sW0[tid] = gw0[tid];
+#pragma unroll 1
+      for (int e = tid; e < L * kW; e += kThreads) sB[e] = gb[e];
+      if (tid < kW) sWo[tid] = gwo[tid];
+      if (tid == 0) sBo[0] = gbo[0];
       fence_proxy_async();
       __syncthreads();
       loaded = k;
@@ -800,8 +805,7 @@ cudaError_t launch_t(const QueryParams &p, int num_sms, int ctas_per_sm, cudaStr
     if (pairs < grid) grid = pairs;
   }
   if (grid < 1) grid = 1;
-  query_w64_kernel<kF16><<<(int)grid, kThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_overlapped(query_w64_kernel<kF16>, dim3((unsigned)grid), kThreads, smem, s, p);
 }
 
 }  // namespace
