@@ -32,9 +32,9 @@
 // reads bounded the kernel at 0.54 of the FMA rate; here the FP32 pipe is busy
 // 0.7 of the time (a paired FMA beside the moves that double a weight runs at
 // 0.75-0.88 of the pipe in a probe; scalar FMAs in this layout measure 3-9%
-// slower).  Measured, before -> now: 131,077 points of 3-512x8-1 22.9 -> 17.8 ms,
-// 300,000 of the 8 x 256 Fourier-feature network 16.8 -> 11.5 ms, 1,048,576 of
-// 3-64x3-1 1.23 -> 0.76 ms, 1,000 points of 3-512x8-1 0.85 -> 0.73 ms.
+// slower).  Measured, before -> now: 131,077 points of 3-512x8-1 22.9 -> 16.9 ms,
+// 300,000 of the 8 x 256 Fourier-feature network 16.8 -> 11.1 ms, 1,048,576 of
+// 3-64x3-1 1.23 -> 0.77 ms, 1,000 points of 3-512x8-1 0.85 -> 0.66 ms.
 // Each accumulator is the same chain of FMAs over k, so z, the activations and
 // the slopes keep their bits.  A layer's output replaces its input in place
 // once every warp has read it, which leaves room for tiles of 64 points at
@@ -66,9 +66,11 @@ struct Cfg {
   static constexpr int THREADS = 32 * CW * PW;
   static constexpr int P = 32 * PW;                     // points per tile
   static constexpr int XS = P + 4;                      // floats per activation row
-  static constexpr int KC = W == 512 ? 8 : (4096 / W > W ? W : 4096 / W);   // panel rows per chunk
+  // panel rows per chunk (at width 512 chunks of 8 rows cost 5-12% more: each chunk
+  // has its barrier and its copies' addresses)
+  static constexpr int KC = W == 512 ? 16 : (4096 / W > W ? W : 4096 / W);
   static constexpr int NCHUNK = W / KC;
-  static constexpr int NS = (W == 512 && PT_ == 8) ? 3 : 2;                 // ring slots
+  static constexpr int NS = 2;                          // ring slots
   // CTAs per SM that the registers are budgeted for
   static constexpr int MIN_CTAS = THREADS >= 512 ? 1 : (W >= 128 ? 512 / THREADS : 768 / THREADS);
   static_assert(W % (8 * TC) == 0 && W % KC == 0 && P <= THREADS, "shape");
@@ -190,28 +192,39 @@ __global__ void __launch_bounds__(Cfg<W, PT_>::THREADS, Cfg<W, PT_>::MIN_CTAS)
 
     // ---- the tile's weight panels, in the order they are used, as one stream
     // of KC-row chunks: (ff0_t), fwd_t 1 .. L-1, bwd L-1 .. 1, (ff0) ----
-    const int nchunks = (2 * (L - 1) + (FF ? 2 : 0)) * C::NCHUNK;
-    auto stage = [&](int q) {
-      if (q < nchunks) {
-        int m = q / C::NCHUNK;
-        const float *src;
-        if (FF && m == 0) {
-          src = ff0_t;
-        } else {
-          if (FF) --m;
-          src = m < L - 1 ? fwd_t + (size_t)m * W * W
-                          : (m < 2 * (L - 1) ? bwdw + (size_t)(2 * (L - 1) - 1 - m) * W * W : ff0);
+    const int npanels = 2 * (L - 1) + (FF ? 2 : 0);
+    int next_panel = 0, next_chunk = 0;          // what stage() copies next
+    const float4 *next_src = nullptr;
+    auto stage = [&](int slot_index) {
+      if (next_panel < npanels) {
+        if (next_chunk == 0) {
+          int m = next_panel;
+          const float *src;
+          if (FF && m == 0) {
+            src = ff0_t;
+          } else {
+            if (FF) --m;
+            src = m < L - 1 ? fwd_t + (size_t)m * W * W
+                            : (m < 2 * (L - 1) ? bwdw + (size_t)(2 * (L - 1) - 1 - m) * W * W : ff0);
+          }
+          next_src = reinterpret_cast<const float4 *>(src) + tid;
         }
-        const float4 *s4 = reinterpret_cast<const float4 *>(src + (size_t)(q % C::NCHUNK) * C::KC * W);
-        float4 *d4 = reinterpret_cast<float4 *>(Ms + (q % C::NS) * C::KC * W);
-#pragma unroll 4
-        for (int v = tid; v < C::KC * W / 4; v += C::THREADS) cp_async16(d4 + v, s4 + v);
+        float4 *dst = reinterpret_cast<float4 *>(Ms + slot_index * C::KC * W) + tid;
+        constexpr int kCopies = C::KC * W / 4 / C::THREADS;
+        static_assert(C::KC * W / 4 % C::THREADS == 0, "whole copies per thread");
+#pragma unroll
+        for (int v = 0; v < kCopies; ++v) cp_async16(dst + v * C::THREADS, next_src + v * C::THREADS);
+        next_src += C::KC * W / 4;
+        if (++next_chunk == C::NCHUNK) {
+          next_chunk = 0;
+          ++next_panel;
+        }
       }
       cp_async_commit();
     };
-    int q = 0;                                   // chunks consumed
-#pragma unroll
-    for (int i = 0; i < C::NS - 1; ++i) stage(i);
+    static_assert(C::NS == 2, "the ring's slots alternate");
+    int q = 0;                                   // slot of the chunk to consume
+    stage(0);
 
     // ---- a1: point load (+ T^{-1}) ----
     if (tid < C::P) {
@@ -241,11 +254,11 @@ __global__ void __launch_bounds__(Cfg<W, PT_>::THREADS, Cfg<W, PT_>::MIN_CTAS)
         for (int h = 0; h < 4; ++h) acc[j][h] = make_float2(0.f, 0.f);
       const float *xk = X + pb;
 #pragma unroll 1
-      for (int kc = 0; kc < C::NCHUNK; ++kc, ++q) {
-        cp_async_wait<C::NS - 2>();
-        __syncthreads();          // chunk q is there, chunk q - 1 and (kc = 0) X are done with
-        stage(q + C::NS - 1);
-        const float *mk = Ms + (q % C::NS) * C::KC * W + cb;
+      for (int kc = 0; kc < C::NCHUNK; ++kc, q ^= 1) {
+        cp_async_wait<0>();
+        __syncthreads();          // this chunk is there; the one before and (kc = 0) X are done with
+        stage(q ^ 1);
+        const float *mk = Ms + q * C::KC * W + cb;
 #pragma unroll 4
         for (int k = 0; k < C::KC; ++k, xk += C::XS, mk += W) {
           const float4 xa = *reinterpret_cast<const float4 *>(xk);
