@@ -3,9 +3,9 @@
 Each step: one explicit Verlet step of the quad mass-spring cloth
 (nsdf_cloth_step), then the collision solve of every vertex against the
 network (nsdf_collide: f < eps moves the vertex to its contact point), written
-in place.  ``ClothSim.run`` times every step with CUDA events.  A brute-force
+in place.  ``ClothSim.run`` times every step with CUDA events.  A
 reference step evaluates the exact mesh SDF of every vertex instead
-(nsdf_mesh_sdf), the plain method the network replaces.
+(nsdf_mesh_sdf), the method the network replaces.
 """
 
 import time
@@ -46,7 +46,7 @@ class ClothSim:
 
 
 def mesh_reference_step_ms(V, F, pts, repeats=3):
-    """Time of the exact brute-force mesh SDF of every vertex (ms per step)."""
+    """Time of the exact mesh SDF of every vertex (ms per step)."""
     Vd = torch.from_numpy(np.asarray(V, np.float32)).cuda().contiguous()
     Fd = torch.from_numpy(np.asarray(F, np.int32)).cuda().contiguous()
     out = torch.empty(pts.shape[0], device="cuda")

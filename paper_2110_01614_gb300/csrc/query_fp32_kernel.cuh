@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(Cfg<W, PT_>::THREADS, Cfg<W, PT_>::MIN_CTAS)
         __syncthreads();          // this chunk is there; the one before and (kc = 0) X are done with
         stage(q ^ 1);
         const float *mk = Ms + q * C::KC * W + cb;
-#pragma unroll 4
+        constexpr int kUnroll = W <= 64 ? 2 : 4;   // (four spill at the narrow widths' 80 registers)
+#pragma unroll kUnroll
         for (int k = 0; k < C::KC; ++k, xk += C::XS, mk += W) {
           const float4 xa = *reinterpret_cast<const float4 *>(xk);
           const float4 xb = *reinterpret_cast<const float4 *>(xk + 16);

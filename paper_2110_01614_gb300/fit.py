@@ -1,7 +1,7 @@
 """Fitting a signed-distance network to a watertight mesh (Sec. 3.1), on the GPU.
 
 Every step: seeded training points (80% near the surface, 20% uniform), exact
-signed-distance targets from the brute-force mesh kernel (nsdf_mesh_sdf),
+signed-distance targets from the exact mesh distance (nsdf_mesh_sdf),
 f and grad f from nsdf_query and their gradients from the hand-written
 nsdf_backward (through the autograd Function), loss = mean |f - d| + lambda *
 mean (||grad f|| - 1)^2, and an Adam update of the packed FP32 weight blob.
@@ -25,7 +25,7 @@ class MeshFit:
     """FP32 fitting with the hand-written backward (L1 + eikonal).
 
     pool_points=None draws fresh seeded training points every step (the
-    targets from the brute-force mesh kernel each time); pool_points=N samples
+    targets from nsdf_mesh_sdf each time); pool_points=N samples
     N points once, as the paper does (Sec. 3.1 samples a fixed set per shape),
     computes their targets once, and draws a seeded batch of n_points from the
     pool every step.
@@ -133,7 +133,7 @@ class MeshFitTC:
 
     As in the paper (Sec. 3.1, Sec. 4.3), the training set is sampled once: a
     pool of seeded points (80% near the surface, 20% uniform) with exact
-    signed distances from the brute-force mesh kernel; every step draws a
+    signed distances from nsdf_mesh_sdf; every step draws a
     seeded batch from the pool, repacks the FP32 weight blob into the
     kernel's 16-bit layouts, takes the gradient of the paper's L1 loss from
     nsdf_l1_grad (tensor-core forward and reverse passes, weight-gradient

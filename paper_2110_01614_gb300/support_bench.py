@@ -1,7 +1,7 @@
 """Timings of the support workloads around the collision query (one JSON line each).
 
 * fit: one fitting step of the 3-64-64-64-1 network to the displaced
-  icosphere (20,480 triangles) with 250,000 points: brute-force mesh SDF
+  icosphere (20,480 triangles) with 250,000 points: exact mesh SDF
   targets + forward + hand-written backward + Adam (Sec. 3.1); fresh seeded
   points every step, and batches drawn from a pool of 1,048,576 points
   sampled once (as the paper samples a fixed set per shape).
@@ -16,7 +16,7 @@
   layers of 256), BF16 tensor cores against the FP32 grouped kernel.
 * cloth: 1024 x 1024 cloth, per-step time of Verlet + collision solve for the
   body-scale network in BF16 / FP16 / FP32 and for the paper's dragon-shaped
-  network in BF16, and of the exact brute-force mesh SDF of every vertex
+  network in BF16, and of the exact mesh SDF of every vertex
   (20,480 triangles) as the plain reference.
 
 * paper_arch: the paper's own network shapes (Sec. 4.3: a Fourier-feature
@@ -33,14 +33,14 @@
   network.
 * cloth_fitted: 100 steps of the 1024 x 1024 cloth dropped onto the displaced
   icosphere represented by a body-scale network fitted to it (BF16 tensor-core
-  fitting), per-step time in BF16 / FP16 / FP32 and of the brute-force mesh
+  fitting), per-step time in BF16 / FP16 / FP32 and of the exact mesh
   SDF of every vertex.
 * voxel: the voxel SDF baseline (Sec. 4.3, Table 1) at N = 256 against the
   fitted body-scale network: build time, memory, query time for 1M points
   and error against the exact signed distance near the surface.
-* kernels: the brute-force mesh SDF (65,536 points x 20,480 triangles, far
+* kernels: the exact mesh SDF (1,048,576 points x 20,480 triangles, far
   from and near the surface) and one 1024 x 1024 cloth step, each alone with
-  L2 flushed before every launch: pairs per second, and the cloth step's
+  L2 flushed before every launch: points per second, and the cloth step's
   bandwidth against the measured copy bandwidth.
 
 Usage: python -m paper_2110_01614_gb300.support_bench [fit penalty grouped grouped_paper cloth
@@ -216,7 +216,7 @@ def bench_cloth(steps=20):
     V, F = synth.displaced_icosphere(level=5, seed=7)
     sim = ClothSim(n=1024)
     ms, _ = mesh_reference_step_ms(V, F, sim.x, repeats=2)
-    res["mesh_bruteforce_sdf_ms_per_step"] = ms
+    res["mesh_sdf_ms_per_step"] = ms
     return res
 
 
@@ -305,7 +305,7 @@ def bench_cloth_fitted(steps=100, fit_steps=300, fp32_steps=100, fitted=None):
     """Cloth of 1024 x 1024 vertices dropped for `steps` explicit steps onto
     the displaced icosphere represented by the body-scale network fitted to
     it (fit_body); per-step time of Verlet + collision solve in BF16, FP16 and
-    FP32, and of the exact brute-force mesh SDF of every vertex."""
+    FP32, and of the exact mesh SDF of every vertex."""
     V, F = synth.displaced_icosphere(level=5, seed=7)
     blob, info = fitted if fitted is not None else fit_body(fit_steps)
     res = {"workload": "cloth_fitted_body", "grid": "1024x1024", "steps": steps,
@@ -322,7 +322,7 @@ def bench_cloth_fitted(steps=100, fit_steps=300, fp32_steps=100, fitted=None):
         if name == "bf16":
             x_final = sim.x
     ms, _ = mesh_reference_step_ms(V, F, x_final, repeats=3)
-    res["mesh_bruteforce_sdf_ms_per_step"] = ms
+    res["mesh_sdf_ms_per_step"] = ms
     return res
 
 
@@ -399,12 +399,11 @@ def events_ms_flushed(fn, reps, flush):
 
 def bench_kernels(mesh_reps=3, cloth_reps=20):
     """The support kernels alone, each against its bound, L2 flushed before
-    every launch: the brute-force mesh SDF (FP32 ALU + MUFU bound; FP64 for
-    undecided winding numbers) of 1,048,576 points against the
+    every launch: the exact mesh SDF of 1,048,576 points against the
     20,480-triangle displaced icosphere, for points far from the surface
-    (uniform in the cube: the FP32 winding number decides) and for fitting
-    targets (80% within ~0.01 of the surface: many take the FP64 winding
-    number), in point-triangle pairs per second (one warm-up launch each);
+    (uniform in the cube: many triangles are about as near) and for fitting
+    targets (80% within ~0.01 of the surface), in points per second (one
+    warm-up launch each);
     and one Verlet step of the 1024 x 1024 cloth (HBM bound: x and x_prev
     read, x_prev written, 48 bytes per vertex; neighbour reads hit the
     caches) against the measured copy bandwidth (three warm-up launches)."""
@@ -422,9 +421,8 @@ def bench_kernels(mesh_reps=3, cloth_reps=20):
         fn = lambda: nsdf_mesh_sdf(Vd, Fd, pts, out)     # noqa: E731
         fn()
         ms = events_ms_flushed(fn, mesh_reps, flush)
-        pairs = n * int(F.shape[0])
         res[f"mesh_sdf_{name}"] = {"points": n, "triangles": int(F.shape[0]), "ms": ms,
-                                   "pairs_per_s": pairs / (ms * 1e-3)}
+                                   "points_per_s": n / (ms * 1e-3)}
     from . import nsdf_cloth_step
     sim_n = 1024
     x = torch.from_numpy(synth.cloth_grid(sim_n)).cuda()
