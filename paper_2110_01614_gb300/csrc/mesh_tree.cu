@@ -38,7 +38,7 @@
 // tests 3.5 ms; hard points by their own warp, points in Morton order, FP32 filters
 // 2.37 ms; spheres before the triangle tests and rays to the nearest side 2.1 ms;
 // hard points from a list, four warps each 0.96 ms (Morton order had put them
-// all into a few warps).
+// all into a few warps); one warp each where the list is long 0.87 ms.
 
 #include "mesh_tree.cuh"
 
@@ -54,7 +54,7 @@ constexpr int kPointBits = 5;            // Morton bits per axis of the points' 
 constexpr int64_t kPointChunk = int64_t(1) << 20;
 constexpr int64_t kHardMax = int64_t(1) << 18;
 constexpr int kHardWarps = 4;            // warps that search one hard point
-constexpr int kHardBlocks = 152 * 8;
+constexpr int kHardBlocks = 152 * 10;    // as many as are resident
 // Leaves a thread visits before its point is a hard one: 32 where points fill
 // the GPU (6 / 12 / 20 / 32 measured 1.54 / 1.22 / 0.99 / 0.89 ms on 250,000
 // fitting points, 48 and 96 more on far points), 4 where a launch has at most a
@@ -750,8 +750,9 @@ __global__ void __launch_bounds__(128) mesh_tree_kernel(const float4 *__restrict
   out[idx] = wind >= 1 ? -d : d;
 }
 
-// The listed points, a block each in turn: out holds the sign and an upper bound
-// of the distance.
+// The listed points: a warp each in turn, or, when they are few, a block each (its
+// warps do not finish together, and half of them would wait at the block's
+// barriers).  out holds the sign and an upper bound of the distance.
 __global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
     const float4 *__restrict__ tri, const float4 *__restrict__ sphere, const float4 *__restrict__ node,
     int leaves, const MeshTreeHeader *__restrict__ hdr, const float4 *__restrict__ pts,
@@ -759,6 +760,18 @@ __global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
     const int64_t *__restrict__ hard_list, unsigned hard_cap) {
   __shared__ unsigned best_bits;
   const unsigned count = min(*hard_count, hard_cap);
+  if (count > 10u * gridDim.x) {
+    for (unsigned i = blockIdx.x * kHardWarps + (threadIdx.x >> 5); i < count;
+         i += gridDim.x * kHardWarps) {
+      const int64_t idx = hard_list[i];
+      const V3<float> p = query_point(pts, grid, idx);
+      const float slack = slack_of(p, hdr), d = out[idx];
+      const float best = warp_search(p, reach_of(d * d * (1.f + 1e-6f), slack), slack, tri, sphere, node,
+                                     leaves, 0u, 1u, nullptr);
+      if ((threadIdx.x & 31u) == 0u) out[idx] = copysignf(sqrtf(best), d);
+    }
+    return;
+  }
   for (unsigned i = blockIdx.x; i < count; i += gridDim.x) {
     const int64_t idx = hard_list[i];
     const V3<float> p = query_point(pts, grid, idx);
