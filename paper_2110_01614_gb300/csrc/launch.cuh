@@ -4,7 +4,8 @@
 // runs; it touches global memory only after wait_for_predecessor(), which returns
 // once the predecessor has finished and its writes are visible.  It calls
 // release_successor() after that, so that no more than one such kernel waits at a
-// time.  Kernels launched the ordinary way are unaffected on either side.  For
+// time.  Its global loads are plain ones: a load marked invariant (__ldg, const
+// __restrict__) might be moved ahead of the wait.  Kernels launched the ordinary way are unaffected on either side.  For
 // kernels of a few microseconds the gap between two launches is a large part of
 // a call.
 #pragma once

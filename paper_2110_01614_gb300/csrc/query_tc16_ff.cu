@@ -60,6 +60,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "launch.cuh"
 #include "nsdf_internal.h"
 #include "tc_ptx.cuh"
 #include "f32x2.cuh"
@@ -388,7 +389,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int L = prm.n_hidden;
   const int G = 2 * L;                         // products per tile
-  const int64_t ntiles = prm.g_nets > 0 ? (int64_t)prm.g_tile_start[prm.g_nets] : (prm.n + kM - 1) / kM;
   const long long budget = prm.wait_budget;
 
   if (threadIdx.x == 0) {
@@ -417,6 +417,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   cluster_sync();      // every CTA's barriers exist before any multicast targets them
   tc_fence_after();
+  wait_for_predecessor();      // nothing above touches global memory
+  release_successor();
+  const int64_t ntiles = prm.g_nets > 0 ? (int64_t)prm.g_tile_start[prm.g_nets] : (prm.n + kM - 1) / kM;
   const uint32_t tmem = *tmem_slot;
   const uint32_t crank = cluster_rank();
   const uint16_t cmask = (uint16_t)((1u << kCluster) - 1u);
@@ -554,15 +557,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int et = threadIdx.x - 32 * kEpiWarp0;     // 0 .. 32 kEpiWarps - 1
         float4 *dst = reinterpret_cast<float4 *>(smem + kOffBias);
         const float4 *bsrc = reinterpret_cast<const float4 *>(bias);
-        for (int i = et; i < L * kW / 4; i += 32 * kEpiWarps) dst[i] = __ldg(bsrc + i);
+        for (int i = et; i < L * kW / 4; i += 32 * kEpiWarps) dst[i] = bsrc[i];   // (plain loads: see launch.cuh)
         dst = reinterpret_cast<float4 *>(smem + kOffFreq);
         for (int i = et; i < kFreq; i += 32 * kEpiWarps)
-          dst[i] = make_float4(2.f * __ldg(ffB + 3 * i), 2.f * __ldg(ffB + 3 * i + 1),
-                               2.f * __ldg(ffB + 3 * i + 2), 0.f);
+          dst[i] = make_float4(2.f * ffB[3 * i], 2.f * ffB[3 * i + 1], 2.f * ffB[3 * i + 2], 0.f);
         dst = reinterpret_cast<float4 *>(smem + kOffWout);
         const float4 *wosrc = reinterpret_cast<const float4 *>(wout);
-        for (int i = et; i < kW / 4; i += 32 * kEpiWarps) dst[i] = __ldg(wosrc + i);
-        bout = __ldg(bo);
+        for (int i = et; i < kW / 4; i += 32 * kEpiWarps) dst[i] = wosrc[i];
+        bout = *bo;
         __syncwarp();
         if (lane == 0) mbar_arrive(w_ready);
         if (!__all_sync(0xffffffffu, mbar_wait(w_ready, w_phase, budget, abort_flag))) {
@@ -732,13 +734,15 @@ cudaError_t launch_t(const QueryParams &p, const NetDevice &net, int num_sms, cu
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kCluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // launch.cuh
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, query_tc16_ff_kernel<kF16, kSave>, p, net.tmap_fwd, net.tmap_bwd);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
