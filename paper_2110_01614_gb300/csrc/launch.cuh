@@ -4,10 +4,13 @@
 // runs; it touches global memory only after wait_for_predecessor(), which returns
 // once the predecessor has finished and its writes are visible.  It calls
 // release_successor() after that, so that no more than one such kernel waits at a
-// time.  Its global loads are plain ones: a load marked invariant (__ldg, const
-// __restrict__) might be moved ahead of the wait.  Kernels launched the ordinary way are unaffected on either side.  For
-// kernels of a few microseconds the gap between two launches is a large part of
-// a call.
+// time, and a kernel with TMEM only once a block barrier has followed its allocation:
+// the successor's CTAs hold what they allocate until this kernel is done, so nothing
+// that this kernel still needs may be left for them to take.  Its global loads are
+// plain ones: a load marked invariant (__ldg, const __restrict__) might be moved
+// ahead of the wait.  Kernels launched the ordinary way are unaffected on either
+// side.  For kernels of a few microseconds the gap between two launches is a large
+// part of a call.
 #pragma once
 
 #include <cuda_runtime.h>

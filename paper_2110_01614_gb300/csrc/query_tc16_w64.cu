@@ -42,7 +42,7 @@
 // in f32x2 pairs and the weights arriving while L0 is computed.  Sums over the
 // 64 columns stay one chain in column order, which the second warpgroup takes
 // over from the first, so both kernels give the same bits.  4,096 points of
-// 3-64x3-1: 17.2 -> 9.6 us a call (12.3 without the overlapped launch).  On large calls (1,048,576 points, grouped
+// 3-64x3-1: 17.2 -> 9.8 us a call (12.3 without the overlapped launch).  On large calls (1,048,576 points, grouped
 // scenes) that form measured 0.90-1.02 of this one's speed, with one or two
 // warpgroups per tile: the epilogues' latency, not their FP32 instructions,
 // bounds them.
@@ -570,6 +570,9 @@ __global__ void __launch_bounds__(256, 1)
                  "r"(ncols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
+  // No warp may release the successor before this CTA holds its columns: a successor
+  // that took them first would wait for this kernel, and this kernel for it.
+  __syncthreads();
   wait_for_predecessor();
   release_successor();
   // everything the tile needs is asked for at once
