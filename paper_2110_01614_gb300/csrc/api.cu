@@ -158,6 +158,12 @@ cudaError_t last_err() { return cudaGetLastError(); }
 
 }  // namespace
 
+// A buffer that grows to the largest call seen.
+struct Scratch {
+  float *p = nullptr;
+  size_t bytes = 0;
+};
+
 struct nsdf_ctx {
   nsdf_arch arch{};
   nsdf_precision prec = NSDF_FP32;
@@ -166,8 +172,10 @@ struct nsdf_ctx {
   int num_sms = 0;
   std::vector<NetDevice> nets;
   std::vector<void *> allocations;
-  float *scratch = nullptr;     // per-CTA slope slabs of the query kernels
-  size_t scratch_bytes = 0;
+  // per-CTA slope slabs of the context's query kernel, and, in a 16-bit context, of
+  // the FP32 kernel beside it (its own buffer: a call of one kernel must not free
+  // what a captured graph of the other addresses)
+  Scratch scratch, scratch32;
   int *d_err = nullptr;         // device error word
   float *bwd_partial = nullptr; // per-CTA weight-gradient partial sums of nsdf_backward
   size_t bwd_partial_bytes = 0;
@@ -222,33 +230,43 @@ bool use_w64(const nsdf_ctx *ctx) {
   return use_bf16(ctx) && ctx->arch.ff_freqs == 0 && ctx->arch.width == 64;
 }
 
-int query_grid(const nsdf_ctx *ctx, int64_t n) {
-  if (use_w64(ctx)) return ctx->num_sms;
-  if (use_tc16_ff(ctx)) return query_tc16_ff_grid(n, ctx->num_sms);
-  if (use_bf16(ctx)) return query_tc16_grid(ctx->arch.width, n, ctx->num_sms);
-  return query_fp32_grid(ctx->arch.width, n, ctx->num_sms, ctx->arch.ff_freqs > 0);
+// CTAs of a 16-bit query over n points.
+int tc16_grid(const nsdf_ctx *ctx, int64_t n) {
+  return use_tc16_ff(ctx) ? query_tc16_ff_grid(n, ctx->num_sms)
+                          : query_tc16_grid(ctx->arch.width, n, ctx->num_sms);
 }
 
-size_t query_scratch(const nsdf_ctx *ctx, int grid) {
+// Scratch of the FP32 kernel for calls of up to n points (n_nets > 0: grouped ones).
+size_t fp32_scratch(const nsdf_ctx *ctx, int64_t n, int n_nets) {
+  return fp32_scratch_bytes(ctx->arch.width, ctx->arch.n_hidden, n, n_nets, ctx->num_sms,
+                            ctx->arch.ff_freqs > 0);
+}
+
+// Scratch of a query over n points; it never falls as n grows (see fp32_scratch_bytes).
+size_t query_scratch(const nsdf_ctx *ctx, int64_t n) {
   if (use_w64(ctx)) return 0;
-  if (use_tc16_ff(ctx)) return query_tc16_ff_scratch_bytes(grid);
-  if (use_bf16(ctx))
-    return query_tc16_scratch_bytes(ctx->arch.width, ctx->arch.n_hidden, grid, ctx->prec == NSDF_FP16);
-  return query_fp32_scratch_bytes(ctx->arch.width, ctx->arch.n_hidden, grid);
+  if (!use_bf16(ctx)) return fp32_scratch(ctx, n, 0);
+  const int grid = tc16_grid(ctx, n);
+  return use_tc16_ff(ctx) ? query_tc16_ff_scratch_bytes(grid)
+                          : query_tc16_scratch_bytes(ctx->arch.width, ctx->arch.n_hidden, grid,
+                                                     ctx->prec == NSDF_FP16);
 }
 
-nsdf_status ensure_scratch(nsdf_ctx *ctx, size_t bytes) {
-  if (bytes <= ctx->scratch_bytes) return NSDF_OK;
-  if (ctx->scratch) cudaFree(ctx->scratch);
-  ctx->scratch = nullptr;
-  ctx->scratch_bytes = 0;
+// The FP32 kernel's buffer.
+Scratch &fp32_buffer(nsdf_ctx *ctx) { return use_bf16(ctx) ? ctx->scratch32 : ctx->scratch; }
+
+nsdf_status ensure_scratch(Scratch &sc, size_t bytes) {
+  if (bytes <= sc.bytes) return NSDF_OK;
+  if (sc.p) cudaFree(sc.p);
+  sc.p = nullptr;
+  sc.bytes = 0;
   void *q = nullptr;
   if (cudaMalloc(&q, bytes) != cudaSuccess) {
     cudaGetLastError();
     return NSDF_ERR_OOM;
   }
-  ctx->scratch = static_cast<float *>(q);
-  ctx->scratch_bytes = bytes;
+  sc.p = static_cast<float *>(q);
+  sc.bytes = bytes;
   return NSDF_OK;
 }
 
@@ -298,7 +316,7 @@ nsdf_status ensure_pipeline(nsdf_ctx *ctx) {
   // chunk ends in a partly filled wave of tiles
   int64_t chunk = 1 << 18;
   if (use_bf16(ctx) && !use_w64(ctx)) {
-    const int64_t wave = (int64_t)query_grid(ctx, chunk) * 128;
+    const int64_t wave = (int64_t)tc16_grid(ctx, chunk) * 128;
     const int64_t waves = (chunk + wave / 2) / wave;
     chunk = (waves > 0 ? waves : 1) * wave;
   }
@@ -318,8 +336,7 @@ nsdf_status ensure_pipeline(nsdf_ctx *ctx) {
     return NSDF_ERR_OOM;
   }
   ctx->stage = static_cast<float *>(q);
-  const int grid = query_grid(ctx, chunk);
-  const size_t sb = query_scratch(ctx, grid);
+  const size_t sb = query_scratch(ctx, chunk);
   for (int i = 0; i < 2; ++i) {
     if (cudaMalloc(&q, sb) != cudaSuccess) {
       cudaGetLastError();
@@ -413,8 +430,8 @@ nsdf_status ctx_query_setup(nsdf_ctx *ctx, QueryParams *p, int *num_sms, int *wi
 nsdf_status ctx_set_transform(const float *T, QueryParams *p) { return set_transform(T, *p); }
 
 nsdf_status ctx_query_scratch(nsdf_ctx *ctx, int64_t n, QueryParams *p) {
-  nsdf_status st = ensure_scratch(ctx, query_scratch(ctx, query_grid(ctx, n)));
-  if (st == NSDF_OK) p->scratch = ctx->scratch;
+  nsdf_status st = ensure_scratch(ctx->scratch, query_scratch(ctx, n));
+  if (st == NSDF_OK) p->scratch = ctx->scratch.p;
   return st;
 }
 
@@ -550,7 +567,8 @@ nsdf_status nsdf_destroy(nsdf_ctx *ctx) {
   if (!ctx) return NSDF_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
   for (void *p : ctx->allocations) cudaFree(p);
-  if (ctx->scratch) cudaFree(ctx->scratch);
+  if (ctx->scratch.p) cudaFree(ctx->scratch.p);
+  if (ctx->scratch32.p) cudaFree(ctx->scratch32.p);
   if (ctx->bwd_partial) cudaFree(ctx->bwd_partial);
   if (ctx->stage) cudaFree(ctx->stage);
   for (int i = 0; i < 2; ++i) {
@@ -634,10 +652,9 @@ nsdf_status nsdf_query(nsdf_ctx *ctx, const float *pts, int64_t n, float *out_n_
   p.out_n_sdf = reinterpret_cast<float4 *>(out_n_sdf);
   p.collide = 0;
   p.raw_gradient = (flags & NSDF_RAW_GRADIENT) ? 1 : 0;
-  const int grid = query_grid(ctx, n);
-  nsdf_status st = ensure_scratch(ctx, query_scratch(ctx, grid));
+  nsdf_status st = ensure_scratch(ctx->scratch, query_scratch(ctx, n));
   if (st != NSDF_OK) return st;
-  p.scratch = ctx->scratch;
+  p.scratch = ctx->scratch.p;
   return map_err(launch_query(ctx, 0, p, s));
 }
 
@@ -667,10 +684,9 @@ nsdf_status nsdf_collide(nsdf_ctx *ctx, const float *pts, int64_t n, float eps, 
   p.out_pts = reinterpret_cast<float4 *>(out_pts);
   p.out_n_sdf = reinterpret_cast<float4 *>(out_n_sdf);
   p.out_hit = out_hit;
-  const int grid = query_grid(ctx, n);
-  st = ensure_scratch(ctx, query_scratch(ctx, grid));
+  st = ensure_scratch(ctx->scratch, query_scratch(ctx, n));
   if (st != NSDF_OK) return st;
-  p.scratch = ctx->scratch;
+  p.scratch = ctx->scratch.p;
   return map_err(launch_query(ctx, 0, p, s));
 }
 
@@ -701,10 +717,10 @@ nsdf_status nsdf_backward(nsdf_ctx *ctx, const float *pts, int64_t n, const floa
     p.n = n;
     p.grad_scale = g_sdf;
     p.out_grad = reinterpret_cast<float4 *>(g_pts);
-    const int grid = query_fp32_grid(a.width, n, ctx->num_sms, a.ff_freqs > 0);
-    nsdf_status st = ensure_scratch(ctx, query_fp32_scratch_bytes(a.width, a.n_hidden, grid));
+    Scratch &sc = fp32_buffer(ctx);
+    nsdf_status st = ensure_scratch(sc, fp32_scratch(ctx, n, 0));
     if (st != NSDF_OK) return st;
-    p.scratch = ctx->scratch;
+    p.scratch = sc.p;
     return map_err(launch_query_fp32(p, ctx->num_sms, s));
   }
   if (a.activation != NSDF_ACT_SOFTPLUS || a.ff_freqs > 0 ||
@@ -778,24 +794,13 @@ nsdf_status grouped_check(nsdf_ctx *ctx, const GroupedArgs &g) {
   return NSDF_OK;
 }
 
-// Grid of a grouped launch for a tile shape and CTAs per SM (0 = as many as fit):
-// enough CTAs for the largest possible work list, at most what is resident.
-int grouped_grid(const nsdf_ctx *ctx, int pt, int cps, int64_t max_total) {
-  const int P = fp32_tile_points(ctx->arch.width, pt);
-  const int fit = fp32_ctas_per_sm(ctx->arch.width, pt, ctx->arch.ff_freqs > 0);
-  if (cps <= 0 || cps > fit) cps = fit;
-  const int64_t max_tiles = (max_total + P - 1) / P + ctx->n_nets;
-  const int64_t cap = (int64_t)ctx->num_sms * cps;
-  return (int)(max_tiles < cap ? max_tiles : cap);
-}
-
 // Grouped launch of the 16-bit Fourier-feature kernel: 128-point tiles, each
 // network's tile count rounded up to even (a 2-CTA cluster takes two tiles of
 // one network at a time).
 nsdf_status grouped_launch_tc16_ff(nsdf_ctx *ctx, const GroupedArgs &g, cudaStream_t s) {
   const int64_t max_tiles = (g.max_total + 127) / 128 + 2 * (int64_t)ctx->n_nets;
   const int grid = query_tc16_ff_grouped_grid(max_tiles, ctx->num_sms);
-  nsdf_status st = ensure_scratch(ctx, query_tc16_ff_scratch_bytes(grid));
+  nsdf_status st = ensure_scratch(ctx->scratch, query_tc16_ff_scratch_bytes(grid));
   if (st != NSDF_OK) return st;
   cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, 128,
                                        g.max_total, ctx->d_tile_start, 2, g.T, ctx->d_body,
@@ -809,7 +814,7 @@ nsdf_status grouped_launch_tc16_ff(nsdf_ctx *ctx, const GroupedArgs &g, cudaStre
   p.eps = g.eps;
   p.out_pts = reinterpret_cast<float4 *>(g.out_pts);
   p.out_n_sdf = reinterpret_cast<float4 *>(g.out_n_sdf);
-  p.scratch = ctx->scratch;
+  p.scratch = ctx->scratch.p;
   p.g_nets = ctx->n_nets;
   p.g_offsets = g.offsets;
   p.g_counts = g.counts;
@@ -848,8 +853,10 @@ nsdf_status grouped_launch(nsdf_ctx *ctx, const GroupedArgs &g, int pt, int cps,
   if (use_tc16_ff(ctx)) return grouped_launch_tc16_ff(ctx, g, s);
   if (use_w64(ctx)) return grouped_launch_w64(ctx, g, cps, s);
   const nsdf_arch &a = ctx->arch;
-  const int grid = grouped_grid(ctx, pt, cps, g.max_total);
-  nsdf_status st = ensure_scratch(ctx, fp32_scratch_bytes_pt(a.width, pt, a.n_hidden, grid));
+  const Fp32Launch l =
+      fp32_grouped_launch(a.width, pt, cps, g.max_total, ctx->n_nets, ctx->num_sms, a.ff_freqs > 0);
+  Scratch &sc = fp32_buffer(ctx);
+  nsdf_status st = ensure_scratch(sc, fp32_scratch(ctx, g.max_total, ctx->n_nets));
   if (st != NSDF_OK) return st;
   cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, fp32_tile_points(a.width, pt),
                                        g.max_total, ctx->d_tile_start, 1, g.T, ctx->d_body,
@@ -863,14 +870,14 @@ nsdf_status grouped_launch(nsdf_ctx *ctx, const GroupedArgs &g, int pt, int cps,
   p.eps = g.eps;
   p.out_pts = reinterpret_cast<float4 *>(g.out_pts);
   p.out_n_sdf = reinterpret_cast<float4 *>(g.out_n_sdf);
-  p.scratch = ctx->scratch;
+  p.scratch = sc.p;
   p.g_nets = ctx->n_nets;
   p.g_offsets = g.offsets;
   p.g_counts = g.counts;
   p.g_tile_start = ctx->d_tile_start;
   p.g_netptrs = ctx->d_netptrs;
   p.g_T = g.T ? ctx->d_body : nullptr;
-  return map_err(launch_query_fp32_grouped(p, pt, grid, s));
+  return map_err(launch_query_fp32_as(p, l, s));
 }
 
 }  // namespace
@@ -990,6 +997,22 @@ nsdf_status nsdf_debug_inject(nsdf_ctx *ctx, int drop_load, long long wait_budge
   if (!ctx || wait_budget_cycles <= 0) return NSDF_ERR_INVALID_ARG;
   ctx->drop_load = drop_load;
   ctx->wait_budget = wait_budget_cycles;
+  return NSDF_OK;
+}
+
+nsdf_status nsdf_debug_fp32_plan(const nsdf_arch *arch, int num_sms, int64_t points, int n_nets,
+                                 int points_per_thread, int ctas_per_sm, int64_t *plan) {
+  if (!arch || !plan || num_sms < 1 || points < 1 || n_nets < 0) return NSDF_ERR_INVALID_ARG;
+  if (!query_fp32_supported(arch->width)) return NSDF_ERR_UNSUPPORTED;
+  if (n_nets > 0 && points_per_thread != 4 && points_per_thread != 8) return NSDF_ERR_INVALID_ARG;
+  const bool ff = arch->ff_freqs > 0;
+  const Fp32Launch l = n_nets == 0 ? fp32_single_launch(arch->width, points, num_sms, ff)
+                                   : fp32_grouped_launch(arch->width, points_per_thread, ctas_per_sm,
+                                                         points, n_nets, num_sms, ff);
+  plan[0] = l.pt;
+  plan[1] = l.grid;
+  plan[2] = (int64_t)fp32_launch_bytes(arch->width, arch->n_hidden, l);
+  plan[3] = (int64_t)fp32_scratch_bytes(arch->width, arch->n_hidden, points, n_nets, num_sms, ff);
   return NSDF_OK;
 }
 

@@ -122,9 +122,9 @@ extern "C" nsdf_status nsdf_collide_noalloc(nsdf_ctx *ctx, const float *pts, int
   // their grid as min(tiles, sm_arg * CTAs per SM), so sm_arg is chosen to
   // keep that product within the slabs the array holds.
   const size_t slab = tc16 ? query_tc16_scratch_bytes(width, n_hidden, 1, fp16)
-                           : query_fp32_scratch_bytes(width, n_hidden, 1);
+                           : fp32_launch_bytes(width, n_hidden, {8, 1});
   const int64_t slabs = (int64_t)(usable_bytes() / slab);
-  const int per_sm = tc16 ? 1 : query_fp32_grid(width, (int64_t)1 << 40, 1, p.ff > 0);
+  const int per_sm = tc16 ? 1 : fp32_ctas_per_sm(width, 8, p.ff > 0);
   if (slabs < per_sm || per_sm < 1) return NSDF_ERR_TOO_LARGE;
   if (tc16 && slabs < query_tc16_min_grid()) return NSDF_ERR_TOO_LARGE;
   int64_t sm_arg = slabs / per_sm;

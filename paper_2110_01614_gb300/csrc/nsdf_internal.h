@@ -116,14 +116,27 @@ bool device_memory(const void *p);
 
 // Launchers (return a cudaError_t from the launch).
 cudaError_t launch_query_fp32(const QueryParams &p, int num_sms, cudaStream_t s);
-size_t query_fp32_scratch_bytes(int width, int n_hidden, int grid);
-int query_fp32_grid(int width, int64_t n, int num_sms, bool ff = false);
 bool query_fp32_supported(int width);
-// grouped FP32 launches with a chosen tile shape (pt = points per thread, 4 or 8)
+// An FP32 launch: tile shape (pt = 4: half the warps and points of pt = 8) and CTAs,
+// each with a slab of scratch for its tile's slopes.
+struct Fp32Launch {
+  int pt, grid;
+};
 int fp32_tile_points(int width, int pt);
 int fp32_ctas_per_sm(int width, int pt, bool ff = false);
-size_t fp32_scratch_bytes_pt(int width, int pt, int n_hidden, int grid);
-cudaError_t launch_query_fp32_grouped(const QueryParams &p, int pt, int grid, cudaStream_t s);
+// of one network over n points
+Fp32Launch fp32_single_launch(int width, int64_t n, int num_sms, bool ff);
+// of many over at most max_total points: enough CTAs for the largest possible work
+// list, at most what is resident (cps CTAs per SM; 0: as many as fit)
+Fp32Launch fp32_grouped_launch(int width, int pt, int cps, int64_t max_total, int n_nets, int num_sms,
+                               bool ff);
+size_t fp32_launch_bytes(int width, int n_hidden, const Fp32Launch &l);   // what it addresses
+// Scratch to hold for calls over up to `points` points: single-network ones (n_nets =
+// 0) or grouped ones of n_nets networks.  Covers every launch of as many points or
+// fewer, in either shape, and never falls as the points grow: a captured graph keeps
+// the buffer's address, so no smaller call may need a larger one.
+size_t fp32_scratch_bytes(int width, int n_hidden, int64_t points, int n_nets, int num_sms, bool ff);
+cudaError_t launch_query_fp32_as(const QueryParams &p, const Fp32Launch &l, cudaStream_t s);
 
 // Weight-gradient products of the fitting loss on the tensor cores
 // (wgrad_tc.cu): for product i, G[gslot[i]] (W x W, row-major [n][k], FP32)

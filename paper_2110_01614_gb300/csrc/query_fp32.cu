@@ -32,31 +32,44 @@ int fp32_ctas_per_sm(int width, int pt, bool ff) {
 }
 
 // Tile shape of a single-network launch: the small tiles when all of them fit
-// on the GPU at once in place of the large ones (more SMs at work; they then
-// also need no more scratch than the large shape's grid), else the large.
-static int single_shape(int width, int64_t n, int num_sms, bool ff) {
-  const int P = fp32_tile_points(width, 4);
-  return (n + P - 1) / P <= (int64_t)num_sms * fp32_ctas_per_sm(width, 8, ff) ? 4 : 8;
-}
-
-int query_fp32_grid(int width, int64_t n, int num_sms, bool ff) {
-  if (!query_fp32_supported(width)) return 0;
-  const int P = fp32_tile_points(width, single_shape(width, n, num_sms, ff));
-  const int64_t tiles = (n + P - 1) / P;
+// on the GPU at once in place of the large ones (more SMs at work), else the large.
+Fp32Launch fp32_single_launch(int width, int64_t n, int num_sms, bool ff) {
+  if (!query_fp32_supported(width)) return {8, 0};
   const int64_t cap = (int64_t)num_sms * fp32_ctas_per_sm(width, 8, ff);
-  return (int)(tiles < cap ? (tiles < 1 ? 1 : tiles) : cap);
+  const int P4 = fp32_tile_points(width, 4), P8 = fp32_tile_points(width, 8);
+  const int64_t tiles4 = (n + P4 - 1) / P4, tiles8 = (n + P8 - 1) / P8;
+  if (tiles4 <= cap) return {4, (int)(tiles4 < 1 ? 1 : tiles4)};
+  return {8, (int)(tiles8 < cap ? tiles8 : cap)};
 }
 
-size_t query_fp32_scratch_bytes(int width, int n_hidden, int grid) {
-  return fp32_scratch_bytes_pt(width, 8, n_hidden, grid);
+Fp32Launch fp32_grouped_launch(int width, int pt, int cps, int64_t max_total, int n_nets, int num_sms,
+                               bool ff) {
+  const int P = fp32_tile_points(width, pt);
+  const int fit = fp32_ctas_per_sm(width, pt, ff);
+  if (cps <= 0 || cps > fit) cps = fit;
+  const int64_t max_tiles = (max_total + P - 1) / P + n_nets;
+  const int64_t cap = (int64_t)num_sms * cps;
+  return {pt, (int)(max_tiles < cap ? max_tiles : cap)};
 }
 
-size_t fp32_scratch_bytes_pt(int width, int pt, int n_hidden, int grid) {
+size_t fp32_launch_bytes(int width, int n_hidden, const Fp32Launch &l) {
   const int slabs = n_hidden > 1 ? n_hidden - 1 : 1;
-  return sizeof(float) * (size_t)grid * slabs * fp32_tile_points(width, pt) * width;
+  return sizeof(float) * (size_t)l.grid * slabs * fp32_tile_points(width, l.pt) * width;
 }
 
-cudaError_t launch_query_fp32_grouped(const QueryParams &p, int pt, int grid, cudaStream_t s) {
+// The bound is taken over both tile shapes and every number of CTAs per SM: `n_nets`
+// tiles beside the points', of the large shape, at most what is resident.
+size_t fp32_scratch_bytes(int width, int n_hidden, int64_t points, int n_nets, int num_sms, bool ff) {
+  const int64_t P4 = fp32_tile_points(width, 4), P8 = fp32_tile_points(width, 8);
+  const int64_t per_sm4 = P4 * fp32_ctas_per_sm(width, 4, ff), per_sm8 = P8 * fp32_ctas_per_sm(width, 8, ff);
+  const int64_t rows = ((points + P8 - 1) / P8 + n_nets) * P8;
+  const int64_t cap = num_sms * (per_sm4 > per_sm8 ? per_sm4 : per_sm8);
+  const int slabs = n_hidden > 1 ? n_hidden - 1 : 1;
+  return sizeof(float) * (size_t)(rows < cap ? rows : cap) * slabs * width;
+}
+
+cudaError_t launch_query_fp32_as(const QueryParams &p, const Fp32Launch &l, cudaStream_t s) {
+  const int pt = l.pt, grid = l.grid;
   if (p.ff > 0) return fp32_ff_launch(p, pt, grid, s);
 #define CASE(W)                                                                           \
   if (p.width == W)                                                                       \
@@ -67,9 +80,9 @@ cudaError_t launch_query_fp32_grouped(const QueryParams &p, int pt, int grid, cu
 }
 
 cudaError_t launch_query_fp32(const QueryParams &p, int num_sms, cudaStream_t s) {
-  const int grid = query_fp32_grid(p.width, p.n, num_sms, p.ff > 0);
-  if (grid == 0) return cudaErrorInvalidValue;
-  return launch_query_fp32_grouped(p, single_shape(p.width, p.n, num_sms, p.ff > 0), grid, s);
+  const Fp32Launch l = fp32_single_launch(p.width, p.n, num_sms, p.ff > 0);
+  if (l.grid == 0) return cudaErrorInvalidValue;
+  return launch_query_fp32_as(p, l, s);
 }
 
 }  // namespace nsdf
