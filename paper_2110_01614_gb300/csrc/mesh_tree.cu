@@ -523,7 +523,11 @@ __device__ float warp_search(V3<float> p, Reach reach, float slack, const float4
       const unsigned ti = t0 + __ffs(tm) - 1;
       tm &= tm - 1;
       if (shared_best) {
-        const float other = __uint_as_float(*(volatile unsigned *)shared_best);
+        // read once for the whole warp: the other warps lower it meanwhile, and lanes
+        // that saw different values would part before the next ballot
+        unsigned bits = 0u;
+        if (lane == 0u) bits = *(volatile unsigned *)shared_best;
+        const float other = __uint_as_float(__shfl_sync(0xffffffffu, bits, 0));
         if (other < best) {
           best = other;
           const Reach closer = reach_of(best, slack);
