@@ -756,7 +756,8 @@ __global__ void __launch_bounds__(128) mesh_tree_kernel(const float4 *__restrict
 
 // The listed points: a warp each in turn, or, when they are few, a block each (its
 // warps do not finish together, and half of them would wait at the block's
-// barriers).  out holds the sign and an upper bound of the distance.
+// barriers).  out holds the sign and an upper bound of the distance, which stays
+// where the search finds nothing (no triangle whose distance FP32 can hold).
 __global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
     const float4 *__restrict__ tri, const float4 *__restrict__ sphere, const float4 *__restrict__ node,
     int leaves, const MeshTreeHeader *__restrict__ hdr, const float4 *__restrict__ pts,
@@ -772,7 +773,7 @@ __global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
       const float slack = slack_of(p, hdr), d = out[idx];
       const float best = warp_search(p, reach_of(d * d * (1.f + 1e-6f), slack), slack, tri, sphere, node,
                                      leaves, 0u, 1u, nullptr);
-      if ((threadIdx.x & 31u) == 0u) out[idx] = copysignf(sqrtf(best), d);
+      if ((threadIdx.x & 31u) == 0u) out[idx] = copysignf(fminf(sqrtf(best), fabsf(d)), d);
     }
     return;
   }
@@ -786,7 +787,8 @@ __global__ void __launch_bounds__(32 * kHardWarps) mesh_hard_kernel(
     warp_search(p, reach_of(d * d * (1.f + 1e-6f), slack), slack, tri, sphere, node, leaves,
                 threadIdx.x >> 5, kHardWarps, &best_bits);
     __syncthreads();
-    if (threadIdx.x == 0) out[idx] = copysignf(sqrtf(__uint_as_float(best_bits)), d);
+    if (threadIdx.x == 0)
+      out[idx] = copysignf(fminf(sqrtf(__uint_as_float(best_bits)), fabsf(d)), d);
     __syncthreads();
   }
 }
