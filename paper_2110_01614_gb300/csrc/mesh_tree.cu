@@ -435,6 +435,10 @@ __device__ __forceinline__ float box_dist2(V3<float> p, float lx, float ly, floa
   return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
+// Below this a square or a product may have lost bits to underflow: such a test is
+// answered the safe way, or in FP64.
+constexpr float kTiny = 1e-36f;
+
 // Is the projected point left of the projected edge, taken upwards (from the
 // end with y <= p.y to the other)?  0 when the edge does not pass p.y.  The
 // sign is the edge's own direction.
@@ -448,7 +452,7 @@ __device__ __forceinline__ int edge_winding(V3<float> p, V3<float> a, V3<float> 
   // left of the edge when (u.x - l.x)(p.y - l.y) > (p.x - l.x)(u.y - l.y);
   // FP32 decides where the products differ by more than their rounding
   const float f = (u.x - l.x) * (p.y - l.y), g = (p.x - l.x) * (u.y - l.y);
-  if (fabsf(f - g) > 1e-6f * (fabsf(f) + fabsf(g))) return f > g ? dir : 0;
+  if (fabsf(f - g) > fmaf(1e-6f, fabsf(f) + fabsf(g), kTiny)) return f > g ? dir : 0;
   const double s = ((double)u.x - l.x) * ((double)p.y - l.y) - ((double)p.x - l.x) * ((double)u.y - l.y);
   return s > 0.0 ? dir : 0;
 }
@@ -462,7 +466,8 @@ __device__ __forceinline__ float plane_side(V3<float> p, V3<float> a, V3<float> 
   const float s = (x1 - x2) * w.x + (y1 - y2) * w.y + (z1 - z2) * w.z;
   const float m = (fabsf(x1) + fabsf(x2)) * fabsf(w.x) + (fabsf(y1) + fabsf(y2)) * fabsf(w.y) +
                   (fabsf(z1) + fabsf(z2)) * fabsf(w.z);
-  if (fabsf(s) > 2e-6f * m) return s;
+  // (an underflowed x, y or z is off by a denormal, times w)
+  if (fabsf(s) > fmaf(2e-6f, m, kTiny * (1.f + fabsf(w.x) + fabsf(w.y) + fabsf(w.z)))) return s;
   const V3<double> du = {(double)b.x - a.x, (double)b.y - a.y, (double)b.z - a.z};
   const V3<double> dv = {(double)c.x - a.x, (double)c.y - a.y, (double)c.z - a.z};
   const V3<double> dw = {(double)a.x - p.x, (double)a.y - p.y, (double)a.z - p.z};
@@ -490,12 +495,12 @@ struct Reach {
 };
 __device__ __forceinline__ Reach reach_of(float best, float slack) {
   const float r = (sqrtf(best) + slack) * (1.f + 1e-6f);
-  return {r, fminf(r * r, kFarDist2)};
+  return {r, fminf(fmaf(r, r, kTiny), kFarDist2)};
 }
 // Can the triangle in sphere s be within reach of p?
 __device__ __forceinline__ bool near_sphere(V3<float> p, const float4 &s, const Reach &reach) {
   const float dx = p.x - s.x, dy = p.y - s.y, dz = p.z - s.z, r = reach.r + s.w;
-  return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= r * r;
+  return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= fmaf(r, r, kTiny);
 }
 
 // One point's search by `warps` warps, of which this is number `warp`: the tree
@@ -602,7 +607,7 @@ __device__ int ray_crossings(V3<float> p0, int dir, const float4 *__restrict__ t
     for (int i = 0; i < kLeaf; ++i) {
       const V3<float> m = along_z<A>({c[i].x, c[i].y, c[i].z});
       const float dx = p.x - m.x, dy = p.y - m.y;
-      if (!(fmaf(dx, dx, dy * dy) <= c[i].w * c[i].w)) continue;
+      if (!(fmaf(dx, dx, dy * dy) <= fmaf(c[i].w, c[i].w, kTiny))) continue;
       const Tri q = load_tri(tri + 3 * (f + i));
       const V3<float> a = along_z<A>(q.a), b = along_z<A>(q.b), d = along_z<A>(q.c);
       const int wn = edge_winding(p, a, b) + edge_winding(p, b, d) + edge_winding(p, d, a);

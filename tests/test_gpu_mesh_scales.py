@@ -1,5 +1,6 @@
-"""The mesh distance at sizes where products of FP32 coordinates overflow: the
-answers of the brute-force kernel."""
+"""The mesh distance at sizes where products of FP32 coordinates overflow or
+underflow: the answers of the brute-force kernel, and signs that do not depend on
+the unit of length (a scale by a power of two is exact)."""
 
 import numpy as np
 import pytest
@@ -60,3 +61,18 @@ def test_no_computable_distance_is_not_infinite(nsdf, radius, n):
     tree, brute = distances(nsdf, V, F, P)
     assert np.isfinite(brute).all()
     np.testing.assert_allclose(np.abs(tree), np.abs(brute), rtol=4 * 2.0 ** -23)
+
+
+@pytest.mark.parametrize("power", [-30, -40, -44, -48, -56, -64])
+def test_signs_do_not_depend_on_the_unit(nsdf, power):
+    V, F = synth.displaced_icosphere(level=3, seed=7)
+    V = V.astype(np.float32)
+    P = points(20000, False)
+    near = V[F[:, 0]] * np.float32(0.999)
+    P[-len(near):, :3] = near
+    ref = distances(nsdf, V, F, P)[0]
+    s = np.float32(2.0 ** power)
+    P[:, :3] *= s
+    got = distances(nsdf, V * s, F, P)[0]
+    assert 0.02 < np.signbit(ref).mean() < 0.98
+    np.testing.assert_array_equal(np.signbit(got), np.signbit(ref))
