@@ -26,13 +26,6 @@ constexpr int kThreads = 256;
 constexpr int kP = 32;                      // points per tile
 constexpr float kInvSqrt2 = 0.70710678118654752f;
 
-__device__ __forceinline__ void sp_and_slope(float z, float beta, float &h, float &s) {
-  const float e = expf(-beta * fabsf(z));
-  h = fmaxf(z, 0.0f) + log1pf(e) / beta;
-  const float inv = 1.0f / (1.0f + e);
-  s = (z >= 0.0f) ? inv : e * inv;
-}
-
 // Shared-memory carve-up (floats), identical on host and device.
 struct BwdLayout {
   int W, L;
@@ -118,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) backward_kernel(const BwdParams prm)
           }
         }
         float h, s;
-        sp_and_slope(z, beta, h, s);
+        softplus_and_slope(z, beta, h, s);
         const float hd = s * zd;
         S[(size_t)l * kP * W + idx] = s;
         ZD[(size_t)l * kP * W + idx] = zd;

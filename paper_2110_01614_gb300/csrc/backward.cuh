@@ -23,6 +23,16 @@ struct BwdParams {
   int out[kBwdMaxL + 1];
 };
 
+// softplus_beta(z) and its slope to FP32 rounding: gradients of networks of any
+// sharpness go through here (the hardware approximations that the query kernel takes
+// err by up to 2^-21 / beta and lose log1p(e) altogether below e = 6e-8).
+__device__ __forceinline__ void softplus_and_slope(float z, float beta, float &h, float &s) {
+  const float e = expf(-beta * fabsf(z));
+  h = fmaxf(z, 0.0f) + log1pf(e) / beta;
+  const float inv = 1.0f / (1.0f + e);
+  s = (z >= 0.0f) ? inv : e * inv;
+}
+
 // Width 64, two or three hidden layers.
 bool backward_w64_supported(int width, int n_hidden);
 cudaError_t launch_backward_w64(const BwdParams &p, int grid, cudaStream_t s);

@@ -22,9 +22,10 @@
 //
 // Bound: the FP32 pipe (50 K FMA a point with both streams: 0.33 ms for 250,000
 // points at its rate).  Measured, 250,000 points of 3-64-64-64-1 with weight
-// gradients: general kernel 3.4 ms, this one 0.62 ms (0.64 with eight point pairs
-// and four columns per warp, whose shared loads take ten wavefronts a k step
-// where this mapping takes six).
+// gradients: general kernel 3.45 ms, this one 0.66 ms (0.61 with the hardware's
+// approximate exp, log and quotient, whose error grows with 1 / beta; 0.76 with IEEE
+// quotients).  Eight point pairs and four columns per warp, whose shared loads take ten
+// wavefronts a k step where this mapping takes six, cost 3%.
 
 #include "backward.cuh"
 #include "f32x2.cuh"
@@ -56,14 +57,15 @@ struct Map {
   static constexpr int total = red + 16 * kW;
 };
 
-// softplus_beta(z) and its slope, as in the FP32 query kernel.
-__device__ __forceinline__ void softplus_and_slope(float z, float beta, float inv_beta, float &h,
-                                                   float &s) {
-  const float u = __expf(-beta * fabsf(z));
-  const float one_u = 1.0f + u;
-  h = fmaf(__logf(one_u), inv_beta, fmaxf(z, 0.0f));
-  const float inv = __fdividef(1.0f, one_u);
-  s = (z >= 0.0f) ? inv : u * inv;
+// As softplus_and_slope, with the two quotients by a residual step each (Newton's
+// method: 1 + e lies in [1, 2], and inv_beta is beta's reciprocal).
+__device__ __forceinline__ void softplus_and_slope_w64(float z, float beta, float inv_beta, float &h,
+                                                       float &s) {
+  const float e = expf(-beta * fabsf(z)), l = log1pf(e), d = 1.0f + e;
+  const float q = l * inv_beta;
+  h = fmaxf(z, 0.0f) + fmaf(fmaf(-q, beta, l), inv_beta, q);
+  const float r = __fdividef(1.0f, d), inv = fmaf(fmaf(-d, r, 1.0f), r, r);
+  s = (z >= 0.0f) ? inv : e * inv;
 }
 
 // Float offset of 16-byte chunk q of weight row n (rows of all layers in turn).
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float h;
-          softplus_and_slope(acc[j][i].x, beta, inv_beta, h, s[l][j][i]);
+          softplus_and_slope_w64(acc[j][i].x, beta, inv_beta, h, s[l][j][i]);
           zd[l][j][i] = acc[j][i].y;
           x[i] = make_float2(h, s[l][j][i] * acc[j][i].y);
           if (l == L - 1) {
