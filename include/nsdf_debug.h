@@ -65,6 +65,14 @@ nsdf_status nsdf_debug_tc16_one_cta(int enable);
 nsdf_status nsdf_debug_fp32_plan(const nsdf_arch *arch, int num_sms, int64_t points, int n_nets,
                                  int points_per_thread, int ctas_per_sm, int64_t *plan);
 
+/*
+ * The FP32 launch of nsdf_collide_noalloc over `points` points within `bytes` of
+ * scratch: plan[0], plan[1], plan[2] as above (plan[1] = 0: refused).
+ * Host-side only (without a GPU one CTA per SM is assumed).
+ */
+nsdf_status nsdf_debug_noalloc_plan(const nsdf_arch *arch, int num_sms, int64_t points, size_t bytes,
+                                    int64_t *plan);
+
 #ifdef __cplusplus
 }
 #endif

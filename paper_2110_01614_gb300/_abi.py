@@ -74,6 +74,8 @@ SIGNATURES = {
     "nsdf_debug_tc16_one_cta": (_ST, [ctypes.c_int]),
     "nsdf_debug_fp32_plan": (_ST, [ctypes.POINTER(nsdf_arch), ctypes.c_int, _I64, ctypes.c_int,
                                    ctypes.c_int, ctypes.c_int, ctypes.POINTER(_I64)]),
+    "nsdf_debug_noalloc_plan": (_ST, [ctypes.POINTER(nsdf_arch), ctypes.c_int, _I64, ctypes.c_size_t,
+                                      ctypes.POINTER(_I64)]),
 }
 
 _lib = None

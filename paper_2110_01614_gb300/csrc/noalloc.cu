@@ -30,7 +30,7 @@
 namespace nsdf {
 
 // 32 MiB: 36 CTAs for the 512-wide, 8-layer body-scale network in 16 bits
-// (896 KiB of slopes per CTA) and in FP32.
+// (896 KiB of slopes per CTA), 73 in FP32 (448 KiB with the small tile).
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
 
 __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];
@@ -118,24 +118,35 @@ extern "C" nsdf_status nsdf_collide_noalloc(nsdf_ctx *ctx, const float *pts, int
     const cudaError_t e = launch_query_tc16_ff(p, *net, fp16, num_sms, s);
     return e == cudaSuccess ? NSDF_OK : NSDF_ERR_CUDA;
   }
-  // one slab per CTA; as many CTAs as whole slabs fit.  The launchers size
-  // their grid as min(tiles, sm_arg * CTAs per SM), so sm_arg is chosen to
-  // keep that product within the slabs the array holds.
-  const size_t slab = tc16 ? query_tc16_scratch_bytes(width, n_hidden, 1, fp16)
-                           : fp32_launch_bytes(width, n_hidden, {8, 1});
-  const int64_t slabs = (int64_t)(usable_bytes() / slab);
-  const int per_sm = tc16 ? 1 : fp32_ctas_per_sm(width, 8, p.ff > 0);
-  if (slabs < per_sm || per_sm < 1) return NSDF_ERR_TOO_LARGE;
-  if (tc16 && slabs < query_tc16_min_grid()) return NSDF_ERR_TOO_LARGE;
-  int64_t sm_arg = slabs / per_sm;
-  if (sm_arg > num_sms) sm_arg = num_sms;
-  const int ctas = (int)sm_arg;
+  // one slab per CTA; as many CTAs as whole slabs fit
+  Fp32Launch l32{8, 0};
+  int64_t ctas = 0;
+  if (tc16) {
+    ctas = (int64_t)(usable_bytes() / query_tc16_scratch_bytes(width, n_hidden, 1, fp16));
+    if (ctas < query_tc16_min_grid()) return NSDF_ERR_TOO_LARGE;
+    if (ctas > num_sms) ctas = num_sms;
+  } else {
+    l32 = fp32_bounded_launch(width, n_hidden, n, num_sms, p.ff > 0, usable_bytes());
+    if (l32.grid < 1) return NSDF_ERR_TOO_LARGE;
+  }
   void *scratch = nullptr;
   if (scratch_address(&scratch) != cudaSuccess) return NSDF_ERR_CUDA;
   p.scratch = static_cast<float *>(scratch);
-  const cudaError_t e = tc16 ? launch_query_tc16_net(p, *net, fp16, ctas, s)
-                             : launch_query_fp32(p, ctas, s);
+  const cudaError_t e = tc16 ? launch_query_tc16_net(p, *net, fp16, (int)ctas, s)
+                             : launch_query_fp32_as(p, l32, s);
   return e == cudaSuccess ? NSDF_OK : NSDF_ERR_CUDA;
+}
+
+extern "C" nsdf_status nsdf_debug_noalloc_plan(const nsdf_arch *arch, int num_sms, int64_t points,
+                                               size_t bytes, int64_t *plan) {
+  if (!arch || !plan || num_sms < 1 || points < 1) return NSDF_ERR_INVALID_ARG;
+  if (!query_fp32_supported(arch->width)) return NSDF_ERR_UNSUPPORTED;
+  const Fp32Launch l =
+      fp32_bounded_launch(arch->width, arch->n_hidden, points, num_sms, arch->ff_freqs > 0, bytes);
+  plan[0] = l.pt;
+  plan[1] = l.grid;
+  plan[2] = (int64_t)fp32_launch_bytes(arch->width, arch->n_hidden, l);
+  return NSDF_OK;
 }
 
 extern "C" nsdf_status nsdf_debug_noalloc_limit(size_t bytes) {

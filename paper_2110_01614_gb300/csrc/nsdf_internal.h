@@ -130,6 +130,8 @@ Fp32Launch fp32_single_launch(int width, int64_t n, int num_sms, bool ff);
 // list, at most what is resident (cps CTAs per SM; 0: as many as fit)
 Fp32Launch fp32_grouped_launch(int width, int pt, int cps, int64_t max_total, int n_nets, int num_sms,
                                bool ff);
+// of one network over n points, in at most `bytes` of scratch (grid 0: not one slab fits)
+Fp32Launch fp32_bounded_launch(int width, int n_hidden, int64_t n, int num_sms, bool ff, size_t bytes);
 size_t fp32_launch_bytes(int width, int n_hidden, const Fp32Launch &l);   // what it addresses
 // Scratch to hold for calls over up to `points` points: single-network ones (n_nets =
 // 0) or grouped ones of n_nets networks.  Covers every launch of as many points or
