@@ -264,11 +264,12 @@ nsdf_status nsdf_query_grouped_T(nsdf_ctx *ctx, const float *pts,
                                  nsdf_stream stream);
 
 /*
- * Autotuner of the grouped launch: times every tile shape (4 or 8 points per
- * thread) and every CTAs-per-SM count that fits on this exact problem
+ * Autotuner of the grouped launch: times every tile shape (8, or 4 with half
+ * the threads and points) and every CTAs-per-SM count that fits on this exact problem
  * (3 timed launches each, CUDA events), keeps the fastest in the context for
- * later nsdf_query_grouped calls and writes it to chosen[0] (points per
- * thread) and chosen[1] (CTAs per SM) when chosen is not NULL.  16-bit
+ * later nsdf_query_grouped calls and writes it to chosen[0] (tile shape) and
+ * chosen[1] (CTAs per SM) when chosen is not NULL.  Without it, FP32 contexts
+ * take the shape by max_total and the number of networks.  16-bit
  * Fourier-feature contexts have one grouped shape (a 128-point tile per
  * CTA, one CTA per SM, on tensor cores): the problem runs once and chosen
  * receives {0, 1}.  16-bit width-64 contexts (two 128-point tiles per CTA
@@ -284,7 +285,7 @@ nsdf_status nsdf_autotune_grouped(nsdf_ctx *ctx, const float *pts,
                                   int *chosen);
 
 /* Set the grouped launch configuration directly (e.g. from a saved tuning):
- * points_per_thread 4 or 8 (FP32 contexts; 16-bit contexts, whose kernels
+ * points_per_thread, the tile shape, 4 or 8 (FP32 contexts; 16-bit contexts, whose kernels
  * have one tile shape, also accept 0), ctas_per_sm >= 0 (0: as many as fit). */
 nsdf_status nsdf_set_grouped_config(nsdf_ctx *ctx, int points_per_thread,
                                     int ctas_per_sm);

@@ -57,7 +57,7 @@ nsdf_status nsdf_debug_tc16_one_cta(int enable);
 /*
  * The FP32 kernel's launch over `points` points on a GPU of `num_sms` SMs, of one
  * network (n_nets = 0) or grouped over n_nets networks with the given tile shape
- * (4 or 8) and CTAs per SM (0: as many as fit):
+ * (4 or 8; 0: by the networks' average size) and CTAs per SM (0: as many as fit):
  *   plan[0] tile shape, plan[1] CTAs, plan[2] bytes of scratch that they address,
  *   plan[3] bytes that a call reserves.
  * Host-side only (without a GPU one CTA per SM is assumed).

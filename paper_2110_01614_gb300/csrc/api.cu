@@ -194,7 +194,7 @@ struct nsdf_ctx {
   int32_t *d_tile_start = nullptr;
   float *d_body = nullptr;     // [n_nets][kBodyFloats] poses of nsdf_query_grouped_T
   void *train = nullptr;       // buffers of nsdf_l1_grad (train.cu)
-  int grouped_pt = 8;          // points per thread of the FP32 tile (4 or 8)
+  int grouped_pt = 0;          // tile shape of FP32 grouped launches (4 or 8; 0: by size)
   int grouped_cps = 0;         // CTAs per SM (0: as many as fit)
 };
 
@@ -858,7 +858,7 @@ nsdf_status grouped_launch(nsdf_ctx *ctx, const GroupedArgs &g, int pt, int cps,
   Scratch &sc = fp32_buffer(ctx);
   nsdf_status st = ensure_scratch(sc, fp32_scratch(ctx, g.max_total, ctx->n_nets));
   if (st != NSDF_OK) return st;
-  cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, fp32_tile_points(a.width, pt),
+  cudaError_t e = launch_grouped_setup(g.offsets, g.counts, ctx->n_nets, fp32_tile_points(a.width, l.pt),
                                        g.max_total, ctx->d_tile_start, 1, g.T, ctx->d_body,
                                        ctx->d_err, s);
   if (e != cudaSuccess) return map_err(e);
@@ -928,7 +928,7 @@ nsdf_status nsdf_autotune_grouped(nsdf_ctx *ctx, const float *pts, const int64_t
     return NSDF_ERR_CUDA;
   float best = 3.0e38f;
   int best_pt = ctx->grouped_pt, best_cps = ctx->grouped_cps;
-  // FP32 kernel: points per thread (4 or 8) and CTAs per SM; 16-bit width-64
+  // FP32 kernel: tile shape (4 or 8) and CTAs per SM; 16-bit width-64
   // kernel: CTAs per SM (its tiles are 128 points, two per CTA)
   const bool w64 = use_w64(ctx);
   const int pts_opts[2] = {4, 8};
@@ -1004,7 +1004,8 @@ nsdf_status nsdf_debug_fp32_plan(const nsdf_arch *arch, int num_sms, int64_t poi
                                  int points_per_thread, int ctas_per_sm, int64_t *plan) {
   if (!arch || !plan || num_sms < 1 || points < 1 || n_nets < 0) return NSDF_ERR_INVALID_ARG;
   if (!query_fp32_supported(arch->width)) return NSDF_ERR_UNSUPPORTED;
-  if (n_nets > 0 && points_per_thread != 4 && points_per_thread != 8) return NSDF_ERR_INVALID_ARG;
+  if (n_nets > 0 && points_per_thread != 0 && points_per_thread != 4 && points_per_thread != 8)
+    return NSDF_ERR_INVALID_ARG;
   const bool ff = arch->ff_freqs > 0;
   const Fp32Launch l = n_nets == 0 ? fp32_single_launch(arch->width, points, num_sms, ff)
                                    : fp32_grouped_launch(arch->width, points_per_thread, ctas_per_sm,

@@ -126,8 +126,9 @@ int fp32_tile_points(int width, int pt);
 int fp32_ctas_per_sm(int width, int pt, bool ff = false);
 // of one network over n points
 Fp32Launch fp32_single_launch(int width, int64_t n, int num_sms, bool ff);
-// of many over at most max_total points: enough CTAs for the largest possible work
-// list, at most what is resident (cps CTAs per SM; 0: as many as fit)
+// of many over at most max_total points (pt = 0: the shape by their average size):
+// enough CTAs for the largest possible work list, at most what is resident (cps CTAs
+// per SM; 0: as many as fit)
 Fp32Launch fp32_grouped_launch(int width, int pt, int cps, int64_t max_total, int n_nets, int num_sms,
                                bool ff);
 // of one network over n points, in at most `bytes` of scratch (grid 0: not one slab fits)
