@@ -566,6 +566,7 @@ nsdf_status nsdf_create(const nsdf_arch *arch, nsdf_precision prec, int n_nets, 
 nsdf_status nsdf_destroy(nsdf_ctx *ctx) {
   if (!ctx) return NSDF_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
+  mesh_scratch_trim(ctx->device);
   for (void *p : ctx->allocations) cudaFree(p);
   if (ctx->scratch.p) cudaFree(ctx->scratch.p);
   if (ctx->scratch32.p) cudaFree(ctx->scratch32.p);

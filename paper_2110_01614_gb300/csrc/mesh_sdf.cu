@@ -16,6 +16,8 @@
 // angle is ill-conditioned) the warp recomputes w in FP64, all 32 lanes
 // splitting the triangles of one such point at a time.
 
+#include <mutex>
+
 #include "mesh_tree.cuh"
 #include "nsdf_internal.h"
 
@@ -120,7 +122,48 @@ __global__ void __launch_bounds__(kThreads) mesh_sdf_kernel(const float *__restr
   if (idx < n) out[idx] = (w > 0.5f) ? -dist : dist;
 }
 
+// The tree's scratch comes from a stream-ordered pool of the library's own, one per
+// device.  The device's default pool gives its memory back whenever the caller
+// synchronises, and the next call would map it again: 180 us, more than a small call
+// takes.  This one keeps up to kPoolKeep bytes between calls and is emptied when a
+// context is destroyed (mesh_scratch_trim).
+constexpr uint64_t kPoolKeep = uint64_t(64) << 20;
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (!g_pool[dev]) {
+    // another thread may be capturing a stream
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+      if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        g_pool[dev] = pool;
+      else
+        cudaMemPoolDestroy(pool);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  return g_pool[dev];
+}
+
 }  // namespace
+
+void mesh_scratch_trim(int device) {
+  if (device < 0 || device >= kMaxDevices) return;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (g_pool[device]) cudaMemPoolTrimTo(g_pool[device], 0);
+}
 
 cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *faces,
                             int64_t n_faces, const float4 *pts, int64_t n, float *out, int grid_n,
@@ -137,16 +180,17 @@ cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *
       g.h[c] = h[c];
     }
   }
-  // The tree needs scratch memory, taken from the device's stream-ordered pool
-  // and given back behind the kernels.  Without it (none left, or a stream
-  // that is being captured: the graph stays free of allocations) the
-  // brute-force kernel answers alone.
+  // The tree needs scratch memory, taken from the pool and given back behind the
+  // kernels.  Without it (none left, or a stream that is being captured: the graph
+  // stays free of allocations) the brute-force kernel answers alone.
   void *mem = nullptr;
   if (n_faces >= kTreeMinFaces && n_faces <= kTreeMaxFaces) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-        cudaMallocAsync(&mem, mesh_tree_bytes(n_faces, pts ? n : 0, pts ? 0 : n), s) != cudaSuccess)
-      mem = nullptr;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+      const cudaMemPool_t pool = scratch_pool();
+      const size_t bytes = mesh_tree_bytes(n_faces, pts ? n : 0, pts ? 0 : n);
+      if (!pool || cudaMallocFromPoolAsync(&mem, bytes, pool, s) != cudaSuccess) mem = nullptr;
+    }
     if (!mem) cudaGetLastError();
   }
   if (mem) {

@@ -177,6 +177,8 @@ cudaError_t launch_query_w64(const QueryParams &p, bool fp16, int num_sms, int c
 cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *faces,
                             int64_t n_faces, const float4 *pts, int64_t n, float *out, int grid_n,
                             const float *lo, const float *h, cudaStream_t s);
+// Gives back the scratch memory that the mesh distance keeps on a device.
+void mesh_scratch_trim(int device);
 
 bool query_tc16_supported(int width, int n_hidden, int skip);
 bool make_tc16_tmaps(NetDevice &net, int width, int n_hidden, bool fp16);
