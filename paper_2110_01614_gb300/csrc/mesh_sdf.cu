@@ -56,13 +56,16 @@ __device__ void load_chunk(TriChunk &t, const float *__restrict__ V, int64_t nv,
   }
 }
 
+// kAfterTree: launched behind the tree's kernels, and without faces, so that nothing
+// is written, where they have answered.  (As an early return the same test made the
+// loop over the faces 5% slower.)
+template <bool kAfterTree>
 __global__ void __launch_bounds__(kThreads) mesh_sdf_kernel(const float *__restrict__ V, int64_t nv,
                                                             const int32_t *__restrict__ F,
                                                             int64_t nf, const float4 *__restrict__ pts,
                                                             int64_t n, float *__restrict__ out,
                                                             const GridPts grid,
                                                             const MeshTreeHeader *tree) {
-  if (tree && mesh_tree_usable(tree)) return;     // the tree kernel has answered
   extern __shared__ float4 smem4[];
   TriChunk &tc = *reinterpret_cast<TriChunk *>(smem4);
   __shared__ double wacc[kThreads / 32][32];
@@ -70,6 +73,7 @@ __global__ void __launch_bounds__(kThreads) mesh_sdf_kernel(const float *__restr
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   V3<float> p = {0.f, 0.f, 0.f};
   if (idx < n) p = query_point(pts, grid, idx);
+  if (kAfterTree && mesh_tree_usable(tree)) nf = 0;
   float best = kFarDist2, wsum = 0.f;
   for (int64_t f0 = 0; f0 < nf; f0 += kChunk) {
     __syncthreads();
@@ -119,7 +123,7 @@ __global__ void __launch_bounds__(kThreads) mesh_sdf_kernel(const float *__restr
     __syncwarp();
     if (redo) w = (float)(wacc[warp][lane] / (4.0 * 3.14159265358979323846));
   }
-  if (idx < n) out[idx] = (w > 0.5f) ? -dist : dist;
+  if (idx < n && (!kAfterTree || nf > 0)) out[idx] = (w > 0.5f) ? -dist : dist;
 }
 
 // The tree's scratch comes from a stream-ordered pool of the library's own, one per
@@ -169,8 +173,10 @@ cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *
                             int64_t n_faces, const float4 *pts, int64_t n, float *out, int grid_n,
                             const float *lo, const float *h, cudaStream_t s) {
   const size_t smem = sizeof(TriChunk);
-  cudaError_t e = cudaFuncSetAttribute(mesh_sdf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(mesh_sdf_kernel<false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mesh_sdf_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   GridPts g{};
   if (!pts) {
@@ -201,8 +207,9 @@ cudaError_t launch_mesh_sdf(const float *verts, int64_t n_verts, const int32_t *
     }
   }
   const int64_t blocks = (n + kThreads - 1) / kThreads;
-  mesh_sdf_kernel<<<(unsigned)blocks, kThreads, smem, s>>>(
-      verts, n_verts, faces, n_faces, pts, n, out, g, static_cast<const MeshTreeHeader *>(mem));
+  const auto brute = mem ? mesh_sdf_kernel<true> : mesh_sdf_kernel<false>;
+  brute<<<(unsigned)blocks, kThreads, smem, s>>>(verts, n_verts, faces, n_faces, pts, n, out, g,
+                                                 static_cast<const MeshTreeHeader *>(mem));
   e = cudaGetLastError();
   if (mem) {
     const cudaError_t e2 = cudaFreeAsync(mem, s);

@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(kBlock) tree_cell_kernel(const float *__restri
                                                            const MeshTreeHeader *__restrict__ hdr,
                                                            unsigned *hist, uint2 *__restrict__ key,
                                                            unsigned *phist, uint2 *__restrict__ pkey) {
+  if (!mesh_tree_usable(hdr)) return;      // (here and below: an open mesh is not built)
   if (blockIdx.x >= fb) {
     const int64_t i = (int64_t)(blockIdx.x - fb) * kBlock + threadIdx.x;
     if (i >= n) return;
@@ -244,9 +245,11 @@ __global__ void __launch_bounds__(kBlock) tree_cell_kernel(const float *__restri
 
 // Exclusive prefix sums of the cell counts, in place: block 0 the faces',
 // block 1 the points'.  32 cells per thread and round (2^15 cells in one).
-__global__ void __launch_bounds__(1024) tree_scan_kernel(unsigned *hist, int cells, unsigned *phist,
+__global__ void __launch_bounds__(1024) tree_scan_kernel(const MeshTreeHeader *__restrict__ hdr,
+                                                         unsigned *hist, int cells, unsigned *phist,
                                                          int pcells) {
   __shared__ unsigned warp_sum[32];
+  if (!mesh_tree_usable(hdr)) return;
   if (blockIdx.x == 1) {
     hist = phist;
     cells = pcells;
@@ -289,9 +292,11 @@ __global__ void __launch_bounds__(1024) tree_scan_kernel(unsigned *hist, int cel
 // per triangle: a, b, c in turn), and the order in which the points are queried.
 __global__ void __launch_bounds__(kBlock) tree_scatter_kernel(
     const float *__restrict__ V, int64_t nv, const int32_t *__restrict__ F, int64_t nf, unsigned fb,
-    int64_t n, const unsigned *__restrict__ start, const uint2 *__restrict__ key,
+    int64_t n, const MeshTreeHeader *__restrict__ hdr, const unsigned *__restrict__ start,
+    const uint2 *__restrict__ key,
     const unsigned *__restrict__ pstart, const uint2 *__restrict__ pkey, float4 *__restrict__ tri,
     unsigned *__restrict__ order) {
+  if (!mesh_tree_usable(hdr)) return;
   if (blockIdx.x >= fb) {
     const int64_t i = (int64_t)(blockIdx.x - fb) * kBlock + threadIdx.x;
     if (i >= n) return;
@@ -347,6 +352,7 @@ __global__ void __launch_bounds__(kBlock) tree_box_kernel(const float4 *__restri
                                                           float *block_box, MeshTreeHeader *hdr) {
   __shared__ Box sb[kBlock];
   __shared__ bool last;
+  if (!mesh_tree_usable(hdr)) return;
   const int t = threadIdx.x;
   const int per = leaves < kBlock ? leaves : kBlock;       // leaves of this block
   const int64_t leaf = (int64_t)blockIdx.x * per + t;
@@ -838,9 +844,9 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
     const float4 *cp = pts ? pts + c0 : nullptr;
     tree_cell_kernel<<<blocks, kBlock, 0, s>>>(verts, n_verts, faces, n_faces, m.bits, fb, cp, k, hdr,
                                               hist, key, phist, pkey);
-    if (fb > 0) tree_scan_kernel<<<pts ? 2 : 1, 1024, 0, s>>>(hist, cells, phist, pcells);
-    else tree_scan_kernel<<<1, 1024, 0, s>>>(phist, pcells, nullptr, 0);
-    tree_scatter_kernel<<<blocks, kBlock, 0, s>>>(verts, n_verts, faces, n_faces, fb, k, hist, key,
+    if (fb > 0) tree_scan_kernel<<<pts ? 2 : 1, 1024, 0, s>>>(hdr, hist, cells, phist, pcells);
+    else tree_scan_kernel<<<1, 1024, 0, s>>>(hdr, phist, pcells, nullptr, 0);
+    tree_scatter_kernel<<<blocks, kBlock, 0, s>>>(verts, n_verts, faces, n_faces, fb, k, hdr, hist, key,
                                                  phist, pkey, tri, order);
     if (fb > 0) {
       const int64_t bb = m.leaves < kBlock ? 1 : m.leaves / kBlock;
