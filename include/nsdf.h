@@ -327,7 +327,7 @@ nsdf_status nsdf_voxel_collide(const float *grid, int n, const float *lo,
  * negative, Sec. 3.2).  verts: float [n_verts*3]; faces: int32 [n_faces*3],
  * counter-clockwise seen from outside; pts float4; all device pointers (a
  * host array: NSDF_ERR_INVALID_ARG, nothing is launched).
- * A closed mesh of at least 128 faces is answered through a bounding-box tree
+ * A closed mesh of at least 192 faces is answered through a bounding-box tree
  * that each call builds in stream-ordered scratch memory; its winding number is
  * the signed count of the faces a ray crosses.  Other meshes, calls recorded
  * into a CUDA graph and calls for which no scratch memory is left evaluate every

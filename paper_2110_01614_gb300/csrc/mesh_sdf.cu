@@ -1,6 +1,6 @@
 // Exact signed distance to a watertight triangle mesh: the ground truth a
 // network is fitted to (Sec. 3.1) and the plain reference a cloth run can
-// collide against.  Closed meshes of 128 faces and more go through the tree of
+// collide against.  Closed meshes of 192 faces and more go through the tree of
 // mesh_tree.cu; this is the brute force for the others and the dispatch.
 //
 // Per point: unsigned distance = min over triangles of the distance to the

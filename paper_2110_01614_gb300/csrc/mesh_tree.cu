@@ -54,14 +54,16 @@ constexpr int kPointBits = 5;            // Morton bits per axis of the points' 
 constexpr int64_t kPointChunk = int64_t(1) << 20;
 constexpr int64_t kHardMax = int64_t(1) << 18;
 constexpr int kHardWarps = 4;            // warps that search one hard point
-constexpr int kHardBlocks = 152 * 10;    // as many as are resident
+constexpr int kHardPerSm = 10;           // blocks that search hard points: as many as are resident
 // Leaves a thread visits before its point is a hard one: 32 where points fill
 // the GPU (6 / 12 / 20 / 32 measured 1.54 / 1.22 / 0.99 / 0.89 ms on 250,000
-// fitting points, 48 and 96 more on far points), 4 where a launch has at most a
-// few points per block of the hard kernel and one thread's descent is all it
-// waits for (4 / 12 / 32: 200 points x 20,480 triangles 215 / 275 / 389 us, 4,000
-// points 240 / 274 / 364 us).
-constexpr int kLeafBudget = 32, kLeafBudgetFew = 4;
+// fitting points, 48 and 96 more on far points), 4 where one thread's descent is all
+// that a launch waits for (4 / 12 / 32: 200 points x 20,480 triangles 215 / 275 / 389
+// us, 4,000 points 240 / 274 / 364 us).  The line is drawn at so many points per
+// block of the hard kernel (48,640 here; 32 -> 4, far points: 8,000 points x 192
+// triangles 173 -> 123 us, x 20,480 451 -> 274; 30,000 points x 320 193 -> 123; near
+// ones 30,000 x 20,480 300 -> 259, x 320 100 -> 105; at 60,000 near points lose 8-19%).
+constexpr int kLeafBudget = 32, kLeafBudgetFew = 4, kFewPerBlock = 32;
 
 // Scratch layout for a mesh of F faces.
 struct TreeMem {
@@ -814,6 +816,11 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
                              int64_t n_faces, const float4 *pts, int64_t n, float *out,
                              const GridPts &grid, void *mem, cudaStream_t s) {
   const TreeMem m = tree_mem(n_faces, pts ? n : 0, pts ? 0 : n);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int hard_blocks = kHardPerSm * sms;
   char *base = static_cast<char *>(mem);
   MeshTreeHeader *hdr = reinterpret_cast<MeshTreeHeader *>(base + m.header);
   unsigned *hist = reinterpret_cast<unsigned *>(base + m.hist);
@@ -828,7 +835,7 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
   float4 *node = reinterpret_cast<float4 *>(base + m.node);
   float *block_box = reinterpret_cast<float *>(base + m.block_box);
   const int cells = 1 << (3 * m.bits), pcells = 1 << (3 * kPointBits);
-  cudaError_t e = cudaMemsetAsync(base + m.header, 0, m.key - m.header, s);
+  e = cudaMemsetAsync(base + m.header, 0, m.key - m.header, s);
   if (e != cudaSuccess) return e;
   unsigned fb = (unsigned)((n_faces + kBlock - 1) / kBlock);
   tree_bounds_kernel<<<fb < 1024 ? fb : 1024, kBlock, 0, s>>>(verts, n_verts, faces, n_faces, hdr);
@@ -861,9 +868,9 @@ cudaError_t launch_mesh_tree(const float *verts, int64_t n_verts, const int32_t 
     }
     mesh_tree_kernel<<<(unsigned)qb, 128, 0, s>>>(tri, sphere, node, (int)m.leaves, hdr, cp, order,
                                                  count, out + c0, grid,
-                                                 n <= 4 * kHardBlocks ? kLeafBudgetFew : kLeafBudget,
+                                                 n <= kFewPerBlock * (int64_t)hard_blocks ? kLeafBudgetFew : kLeafBudget,
                                                  hard_count, hard, m.hard_cap);
-    mesh_hard_kernel<<<kHardBlocks, 32 * kHardWarps, 0, s>>>(tri, sphere, node, (int)m.leaves, hdr, cp,
+    mesh_hard_kernel<<<hard_blocks, 32 * kHardWarps, 0, s>>>(tri, sphere, node, (int)m.leaves, hdr, cp,
                                                             out + c0, grid, hard_count, hard, m.hard_cap);
     if (!pts) break;
   }

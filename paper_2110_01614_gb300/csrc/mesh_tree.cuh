@@ -25,9 +25,13 @@ __device__ __forceinline__ bool mesh_tree_usable(const MeshTreeHeader *h) {
   return h->boundary == 0ull && h->nonfinite == 0u && h->valid > 0u;
 }
 
-// Meshes below this take the brute-force kernel, whose one launch costs less
-// than the tree's seven; above the maximum 32-bit heap indices would run out.
-constexpr int64_t kTreeMinFaces = 128;
+// Meshes below this take the brute-force kernel: far points, whose descents are
+// long, cost more in a tree of so few faces than its eight launches and the descent
+// save (128 faces, 8,000 and 30,000 points anywhere in the cube: 86 and 88 us by brute
+// force, 103 and 109 through the tree; 192 faces: 125 and 127 against 123 and 131; 256:
+// 165 and 166 against 133 and 140.  Points near the surface gain from 128 on).  Above
+// the maximum 32-bit heap indices would run out.
+constexpr int64_t kTreeMinFaces = 192;
 constexpr int64_t kTreeMaxFaces = int64_t(1) << 28;
 
 // n_points: explicit query points; n_nodes: nodes of a grid (the other is 0).
