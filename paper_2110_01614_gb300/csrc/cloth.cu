@@ -12,11 +12,13 @@
 // Bound: instruction issue and memory alike (48 B per vertex, 50 MB at 1024 x
 // 1024: 7.4 us at 6.8 TB/s).  With an IEEE square root and division per spring
 // (about 60 instructions of 590 per vertex) the issue slots were 77% busy; the
-// reciprocal square root with one Newton step needs 14 and carries the same
-// FP32 rounding.  1024 x 1024, x and x_prev from DRAM: 20.5 -> 16.4 us, 14.1 launched overlapped; tiles of 32 x 8 vertices read
-// 1.3 rows per row written.  Evaluating each spring once, in strips that pass
-// the scalars on by shuffles, measured 15.5 us against 12.4 with everything in L2:
-// the shuffles and the lower occupancy cost more than the springs.
+// approximate reciprocal root with a residual step for the length and one for the
+// quotient needs 16 and rounds alike (the same bits on 1024 x 1024 random cloths).
+// 1024 x 1024, x and x_prev from DRAM: 20.5 -> 14.9 us launched overlapped (14.1 with
+// 1 - rest / |d| from the reciprocal alone, which leaves a force on springs at rest);
+// tiles of 32 x 8 vertices read 1.3 rows per row written.  Evaluating each spring once,
+// in strips that pass the scalars on by shuffles, measured 15.5 us against 12.4 with
+// everything in L2: the shuffles and the lower occupancy cost more than the springs.
 
 #include "launch.cuh"
 #include "nsdf_internal.h"
@@ -26,12 +28,14 @@ namespace {
 
 constexpr int kTileX = 32, kTileY = 8;
 
-// k (|d| - rest) / |d| = k (1 - rest / |d|), 0 for a spring of no length.
+// k (|d| - rest) / |d|, 0 for a spring of no length.  The length by a Newton step on
+// its residual, so that a spring at rest gives exactly 0, and so the quotient.
 __device__ __forceinline__ float spring(float dx, float dy, float dz, float rest, float k) {
   const float d2 = dx * dx + dy * dy + dz * dz;
-  float r = rsqrtf(d2);
-  r = fmaf(0.5f * r, fmaf(-d2 * r, r, 1.0f), r);   // to FP32 rounding
-  return d2 > 0.f ? k * fmaf(-rest, r, 1.0f) : 0.f;
+  const float r = rsqrtf(d2), l = d2 * r;
+  const float len = fmaf(0.5f * r, fmaf(-l, l, d2), l);
+  const float a = k * (len - rest), q = a * r;
+  return d2 > 0.f ? fmaf(fmaf(-q, len, a), r, q) : 0.f;
 }
 
 // (Plain pointers: an invariant load might move ahead of the wait.)
