@@ -24,8 +24,14 @@ class SDFQuery(torch.autograd.Function):
         nsdf_query(net.ctx, pts, out, NSDF_RAW_GRADIENT)
         # an FP32 context's grad f serves the first-order point gradient as it is:
         # 16 bytes a point kept instead of a second pass through the network
-        # (1,048,576 vertices of 3-64x3-1: 1.61 -> 0.86 ms, forward and backward)
-        ctx.save_for_backward(pts, out if net.precision == NSDF_FP32 else None)
+        # (1,048,576 vertices of 3-64x3-1: 1.61 -> 0.86 ms, forward and backward).
+        # Nothing is kept where a gradient of the blob will need that pass anyway; the
+        # outputs of a single point are views of `out`, so a copy stays behind.
+        keep = None
+        if (net.precision == NSDF_FP32 and ctx.needs_input_grad[0]
+                and not ctx.needs_input_grad[1]):
+            keep = out if out.shape[0] > 1 else out.clone()
+        ctx.save_for_backward(pts, keep)
         ctx.net = net
         return out[:, 3].contiguous(), out[:, :3].contiguous()
 
@@ -34,8 +40,7 @@ class SDFQuery(torch.autograd.Function):
         pts, f_grad = ctx.saved_tensors
         net = ctx.net
         n = pts.shape[0]
-        if (f_grad is not None and g_f is not None and g_grad is None
-                and ctx.needs_input_grad[0] and not ctx.needs_input_grad[1]):
+        if f_grad is not None and g_f is not None and g_grad is None:
             g_p = f_grad * g_f.detach()[:, None]       # dL/dp = g_f grad f
             g_p[:, 3] = 0.0
             return g_p, None, None
