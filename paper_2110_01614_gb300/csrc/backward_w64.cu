@@ -385,21 +385,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (rc < prm.out[0])
       for (int k = 0; k < 3; ++k) dst[prm.woff[0] + 3 * rc + k] = t_w0[k];
   }
-  // w_out over the 16 point groups, b_out over the 64 points
+  // w_out over the 16 point groups, b_out over the 64 points (a tree: one chain of 64
+  // sums loses the small ones)
 #pragma unroll
   for (int j = 0; j < 4; ++j) sm[M::red + pg * kW + 4 * cg + j] = t_wout[j];
-  if (tid < kP) sm[M::av + tid] = t_a;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t_a += __shfl_xor_sync(0xffffffffu, t_a, o);
+  if (lane == 0 && warp < kP / 32) sm[M::av + warp] = t_a;
   __syncthreads();
   if (tid < kW) {
     float t = 0.f;
     for (int g = 0; g < 16; ++g) t += sm[M::red + g * kW + tid];
     dst[prm.woff[L] + tid] = t;
   }
-  if (tid == 0) {
-    float t = 0.f;
-    for (int p = 0; p < kP; ++p) t += sm[M::av + p];
-    dst[prm.boff[L]] = t;
-  }
+  if (tid == 0) dst[prm.boff[L]] = sm[M::av] + sm[M::av + 1];
 }
 
 template <int L>
