@@ -253,7 +253,7 @@ def nsdf_l1_grad(ctx, pts, targets, g_weights, loss=None, stream=None):
 
 def nsdf_autotune_grouped(ctx, pts, offsets, counts, max_total, eps, out_pts, out_n_sdf=None,
                           stream=None):
-    """Time the grouped launch's tile shapes on this problem; returns (points/thread, CTAs/SM)."""
+    """Time the grouped launch's tile shapes on this problem; returns (tile shape, CTAs/SM)."""
     _work_list(pts, offsets, counts, max_total, out_pts, out_n_sdf)
     chosen = (ctypes.c_int * 2)()
     _check(library().nsdf_autotune_grouped(ctx, _ptr(pts), _ptr(offsets), _ptr(counts),

@@ -772,8 +772,8 @@ struct GroupedArgs {
 };
 
 // Above 2^34 points (275 GB of float4 records, more than the GPU holds) the
-// device-built tile list could pass 2^31 tiles of the smallest (16-point)
-// tile shape and overflow its int32 starts.
+// device-built tile list could pass 2^31 tiles and overflow its int32 starts (2^29
+// of the smallest, 32-point tile shape).
 constexpr int64_t kMaxGroupedPoints = int64_t(1) << 34;
 
 nsdf_status grouped_check(nsdf_ctx *ctx, const GroupedArgs &g) {

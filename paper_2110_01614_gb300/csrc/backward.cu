@@ -286,7 +286,7 @@ cudaError_t launch_backward(const float4 *pts, int64_t n, const float *a, const 
   cudaError_t e;
   // Width 64 with two or three hidden layers: the register-blocked kernel
   // (backward_w64.cu), at every batch size.  One fitting gradient of 250,000
-  // points on 3-64-64-64-1, the query and the loss included: 3.92 -> 0.94 ms.
+  // points on 3-64-64-64-1, the query and the loss included: 3.90 -> 0.99 ms.
   // Other shapes that fit shared memory take the general kernel.
   if (backward_w64_supported(width, n_hidden)) {
     e = launch_backward_w64(p, grid, s);

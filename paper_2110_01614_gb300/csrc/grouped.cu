@@ -6,9 +6,9 @@
 // tile_start[k] = sum_{j<k} ceil(counts[j] / P), and tile t belongs to the
 // network k with tile_start[k] <= t < tile_start[k+1].  The FP32 fused query
 // kernel then walks the tiles persistently, fetching each tile's network
-// weights from a device table of per-network pointers.  The tile shape (points
-// per thread, hence points per tile) and the CTAs per SM come from the
-// context's tuned configuration (nsdf_autotune_grouped).
+// weights from a device table of per-network pointers.  The tile shape and the
+// CTAs per SM come from the context's tuned configuration (nsdf_autotune_grouped)
+// or, without one, from the bodies' average size (query_fp32.cu).
 
 #include "launch.cuh"
 #include "nsdf_internal.h"

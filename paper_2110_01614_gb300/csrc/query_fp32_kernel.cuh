@@ -1,7 +1,7 @@
 // FP32 CUDA-core form of the fused collision query.
 //
-// One persistent CTA (256 threads) walks tiles of P points.  For each tile it
-// runs, without leaving the SM:
+// A persistent CTA (64 to 512 threads, by the width and the tile shape) walks tiles of
+// P points.  For each tile it runs, without leaving the SM:
 //   * L0 (K = 3) on CUDA cores,
 //   * the hidden layers z_l = W_l x_l + b_l, h_l = softplus_beta(z_l) (Eq. 1)
 //     as register-blocked products against weight panels staged in shared
@@ -43,8 +43,9 @@
 // layers' epilogues, with one barrier per chunk.
 //
 // The small shape (PT = 4, half the warps and half the points per tile) is for
-// launches whose small tiles all fit on the GPU at once, where a larger tile
-// would leave SMs idle, and for the grouped launch's tuner.
+// launches whose small tiles all fit on the GPU at once, where a larger tile would
+// leave SMs idle, for grouped launches of small bodies, and for calls whose scratch
+// holds too few of the large tile's slabs (the rules are in query_fp32.cu).
 
 #pragma once
 

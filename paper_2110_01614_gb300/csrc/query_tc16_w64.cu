@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       if (round != prm.drop_load) mma_commit(bar);
     }
     ++round;
-        // one warp waits (asleep between tests), the others at the barrier: 128 polling
+    // one warp waits (asleep between tests), the others at the barrier: 128 polling
     // threads took issue slots from the other tiles (up to 1.5% of the time)
     const bool done = wg_all(wg, r >= 32 || mbar_wait<true>(bar, phase, budget, &no_abort));
     if (done) phase ^= 1u;
@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(256, 1)
     ++round;
   };
   auto done = [&]() -> bool {          // the same for every thread
-        const bool ok =
+    const bool ok =
         __syncthreads_and(tid >= 32 || mbar_wait<true>(bar, phase, budget, &no_abort) ? 1 : 0) != 0;
     if (ok) phase ^= 1u;
     tc_fence_after();

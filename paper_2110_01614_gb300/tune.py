@@ -36,7 +36,7 @@ def tuned_grouped(net, pts, offsets, counts, max_total, eps, out_pts, out_n_sdf=
                   path=DEFAULT_CACHE, retune=False):
     """Apply the cached configuration for this problem, tuning (and caching) it if absent.
 
-    Returns (points per thread, CTAs per SM).  Tuning runs the problem a few
+    Returns (tile shape, CTAs per SM).  Tuning runs the problem a few
     times and synchronises; call it outside CUDA-graph capture.
     """
     cache = load(path)
