@@ -13,7 +13,7 @@
 // The array is kNoAllocScratchBytes large; every GPU that loads the library
 // holds it until the process exits.  The kernels' scratch is one slab per
 // CTA, so the launch uses as many CTAs as there are whole slabs in the array
-// (at most one per SM): larger networks get fewer CTAs and run slower, and a
+// (at most what is resident): larger networks get fewer CTAs and run slower, and a
 // network whose single slab exceeds the array is rejected with
 // NSDF_ERR_TOO_LARGE.  Slabs need no clearing: each tile writes its slopes
 // before reading them.  All calls share the array: calls whose kernels can
